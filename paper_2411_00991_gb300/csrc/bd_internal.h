@@ -11,6 +11,7 @@ constexpr int kMaxShapes = 4;       // patch shapes: full, right, bottom, corner
 constexpr int kMaxL = 63;           // largest PSF side
 constexpr int kMaxS = 64;           // largest stride (prior patch side)
 constexpr int kMaxSlots = 64;       // sweeps per sweep-kernel launch
+constexpr int kLgamma = 1024;       // photon counts with a tabulated log phi!
 constexpr int kRedThreads = 256;    // fixed block size of every reduction
 
 // device error flag bits
@@ -60,6 +61,7 @@ struct Image {
     const float* Ke32;
     int sample_every, n_samples;     // kept objects: every sample_every-th sweep past burn-in, n_samples slots
     const double* adapt_fac;         // [burn_in][2] proposal-scale factors after accept / reject, or null
+    const double* lgam;              // log phi! of the first kLgamma photon counts (augmented problems), or null
 };
 
 // One chain (an instance of a problem with its own state and random stream).
@@ -115,6 +117,8 @@ struct SweepArgs {
                                      // engine, the next round's while the current one computes; 0: none
     int lean;                        // 1: the lean float form (fewer window cells in flight per thread, a
                                      // 64-register budget, more resident warps); same results
+    const void* rmaps;               // row-run form: the launch's window tensor maps, kRowMapBytes per chain
+    int row_vg;                      // row-run form: classes scored at once by one team
 };
 
 // Window staging (float marginal sampler on the camera grid).  The window of
@@ -238,6 +242,41 @@ __host__ __device__ inline SmemPlan smem_plan(int L, int f, int S, int n_tw, int
     return p;
 }
 
+// Row-run form (bd_rows.cu).  A block of G update teams, each scoring VG
+// classes at once, takes runs of up to V = G VG consecutive classes of one
+// class row.  Progress words carry the
+// steps finished (19 bits: at most 64 sweeps x (64^2 + 1) steps a launch) above
+// a count of the runs that changed data, modulo 2^13.
+constexpr int kRowMaxV = 16;         // classes per run (ring slots of one patch-run)
+constexpr int kRowChgBits = 13;
+constexpr uint32_t kRowChgMask = (1u << kRowChgBits) - 1u;
+constexpr int kRowMapBytes = 384;    // three TMA tensor maps per chain: mu, then cumulants or photon counts
+// columns of a run's window box: L + V - 1 cells from a start rounded down to
+// a multiple of 4 cells; a box side is at most 256 elements, 4 per cell
+__host__ __device__ inline int rows_box_w(int L, int V) { return (L + V + 5) & ~3; }
+__host__ __device__ inline int rows_ring_slots(int V) { return V <= 4 ? 4 : V <= 8 ? 8 : 16; }
+struct RowsSmem {
+    size_t K, tw, ent, ring, red, mu, cum, cum2, spec, total;
+};
+__host__ __device__ inline RowsSmem rows_smem(int L, int S, int V, int G, int nwt, int n_tw, int nhalf0, bool aug,
+                                              int spec_entries)
+{
+    RowsSmem p;
+    size_t o = 0;
+    const size_t cells = (size_t)rows_box_w(L, V) * L;
+    p.mu = o; o += al128(4 * cells);
+    p.cum = o; o += al128((aug ? 4 : 16) * cells);
+    p.cum2 = o; o += aug ? 0 : al128(8 * cells);
+    p.K = o; o += al16((size_t)L * L * 4);
+    p.tw = o; o += al16((size_t)n_tw * 8);
+    p.ent = o; o += al16((size_t)nhalf0 * 8);
+    p.ring = o; o += 64 * 16;
+    p.red = o; o += al16((size_t)2 * nwt * 3 * (V + G) * 4);
+    p.spec = o; o += al16((size_t)spec_entries * 8);
+    p.total = o;
+    return p;
+}
+
 // host launchers (defined in the .cu files)
 void launch_setup(const Image& im, const Image* d_im, const float* w, const float* g,
                   const float* o, const float* v, double gs, double os, double vs,
@@ -253,6 +292,8 @@ template <typename T>
 // density p(w, phi, rho) at the chain's photon counts)
 void launch_refresh(const Image& im, const Chain& ch, double* scratch, int write_state,
                     double* out_logpost, const int* out_index, int* err, cudaStream_t st, int64_t* launches);
+// out[k] = log k!, k < kLgamma
+void launch_lgamma(double* out, cudaStream_t st, int64_t* launches);
 // photon counts of every camera pixel drawn from p(phi | w, mu) with the
 // uniforms of sweep t (the augmented sampler's initial draw)
 template <typename T>
@@ -261,6 +302,8 @@ template <typename T>
 cudaError_t launch_sweep(const SweepArgs& a, int grid, int threads, size_t smem, cudaStream_t st);
 template <typename T>
 int sweep_blocks_per_sm(int threads, size_t smem, bool aug, bool fine, int stg, bool solo, bool lean);
+cudaError_t launch_sweep_rows(const SweepArgs& a, int grid, int threads, size_t smem, cudaStream_t st);
+int rows_blocks_per_sm(bool aug, int vg, int threads, size_t smem);
 // zero every chain's progress words and trace partials
 void launch_reset(const Image* d_imgs, const Chain* d_chains, int n_chains, int n_slots, cudaStream_t st,
                   int64_t* launches);

@@ -381,6 +381,18 @@ template void launch_refresh<double>(const Image&, const Chain&, double*, int, d
                                      int64_t*);
 
 // ------------------------------------------------- photon-count draw -----
+__global__ void k_lgamma(double* out)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < kLgamma) out[k] = lgamma((double)k + 1.0);
+}
+
+void launch_lgamma(double* out, cudaStream_t st, int64_t* launches)
+{
+    k_lgamma<<<(kLgamma + 127) / 128, 128, 0, st>>>(out);
+    ++*launches;
+}
+
 template <typename T>
 __global__ void k_sample_phi(Image im, Chain ch, int t, int* err)
 {

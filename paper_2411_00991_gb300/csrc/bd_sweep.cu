@@ -38,74 +38,9 @@
 #include <mutex>
 
 #include "bd_device.cuh"
+#include "bd_update.cuh"
 
 namespace bd {
-
-// One entry of the patch prior change: X' = X + delta w, with
-//   |X'|^2 - |X|^2 = delta (2 Re(X conj w) + delta)        (|w| = 1)
-// accumulates  wa log(|X'|^2/|X|^2),  mult (|X'| - |X|),  mult |X|.
-// The ratio form q = (|X'|^2 - |X|^2)/|X|^2 is free of cancellation while
-// the coefficient does not shrink much (q > -1/2).  When it shrinks toward
-// zero, q rounds to -1 (log1p = -inf, and with wa < 0 an infinite gain that
-// the exact Eq. 7-8 change never has), so there the log is taken of the
-// ratio |X'|^2/|X|^2 itself, with X' the value an accepted update stores.
-// X' exactly 0 is rejected (the Dirichlet density is singular there).
-template <typename T>
-__device__ __forceinline__ void prior_term(T xr, T xi, T wr, T wi, T delta, T wa, T mult, T& accP, T& accS,
-                                           T& accA, bool& bad)
-{
-    using P = Prec<T>;
-    const T n2 = xr * xr + xi * xi;
-    const T dd = delta * ((T)2 * (xr * wr + xi * wi) + delta);
-    const T rn = fma(delta, wr, xr), in = fma(delta, wi, xi);
-    const T n2n = rn * rn + in * in;
-    if (!(n2n > (T)0)) bad = true;
-    const T mo = P::sqrt(n2), mn = P::sqrt(n2n);
-    const T i2 = P::rcp(n2);
-    const T q = dd * i2;
-    accP += wa * (q > (T)-0.5 ? P::log1p(q) : P::log(n2n * i2));
-    accS += mult * (dd * P::rcp(mn + mo));
-    accA += mult * mo;
-}
-
-// The target (Eq. 9) has a finite density at every state a chain can reach,
-// so a proposal whose log acceptance ratio is not finite (and that is not
-// impossible: mu' <= 0, a zero coefficient) is an arithmetic failure.  It is
-// rejected, the numeric error bit raised, and the first such update recorded
-// for the host: err[2] chain, err[3] pixel, err[8] sweep, dL and dP as
-// doubles at err + 4.
-__device__ __noinline__ void report_nonfinite(int* err, int chain, int m, int t, double dL, double dP)
-{
-    atomicOr(err, kErrRatio);
-    if (atomicCAS(err + 1, 0, 1) == 0) {
-        err[2] = chain;
-        err[3] = m;
-        err[8] = t;
-        double* d = reinterpret_cast<double*>(err + 4);
-        d[0] = dL;
-        d[1] = dP;
-    }
-}
-
-// x mod n for 0 <= x < 2^22 through a float reciprocal (exact after one correction)
-__device__ __forceinline__ int small_mod(int x, int n, float inv_n)
-{
-    int r = x - n * __float2int_rz((float)x * inv_n);
-    r += r < 0 ? n : 0;
-    r -= r >= n ? n : 0;
-    return r;
-}
-
-template <typename T>
-__device__ __forceinline__ void twiddle(const T* tw, const Shape& sh, int kl, int u, int v, T& wr, T& wi)
-{
-    const int k = kl >> 16, l = kl & 0xffff;
-    const T* eh = tw + 2 * (sh.twh_off + small_mod(k * u, sh.ph, sh.inv_ph));
-    const T* ew = tw + 2 * (sh.tww_off + small_mod(l * v, sh.pw, sh.inv_pw));
-    wr = eh[0] * ew[0] - eh[1] * ew[1];
-    wi = eh[0] * ew[1] + eh[1] * ew[0];
-}
-
 
 // Window cell k (0 <= k < Lc^2) of object pixel (i, j): the camera pixel
 // (aa, bb) it weighs on and the entry kw of the effective kernel Ke (Le x Le)
@@ -130,25 +65,6 @@ __device__ __forceinline__ bool win_cell(const Image& im, int i, int j, int k, i
     kw = p * Le + q;
     return k < Lc * Lc && (unsigned)aa < (unsigned)im.H && (unsigned)bb < (unsigned)im.W && (unsigned)p < (unsigned)Le &&
            (unsigned)q < (unsigned)Le;
-}
-
-// a2: the proposal of one update from its Philox counter (m, t, chain, 0):
-// z standard normal (Box-Muller), log u, the log-space move hz = s_m z (s_m
-// the pixel's scale: its adapted one, else the problem's step) and
-// rho' = rho exp(hz); hz is also the Hastings term of the decision.
-template <typename T>
-__device__ __forceinline__ void proposal(const Image& im, const Chain& ch, int m, int t, T r_old, T& hz, T& lu,
-                                         T& r_new, T& delta)
-{
-    using P = Prec<T>;
-    const uint4 x = philox4x32_10(make_uint4((uint32_t)m, (uint32_t)t, (uint32_t)ch.chain, 0u), im.seed_lo,
-                                  im.seed_hi);
-    const T z = P::gauss(uniform23<T>(x.x), uniform23<T>(x.y));
-    const T sm = ch.steps != nullptr ? reinterpret_cast<const T*>(ch.steps)[m] : (T)im.step;
-    hz = sm * z;
-    lu = P::log(uniform23<T>(x.z));
-    r_new = r_old * P::exp(hz);
-    delta = r_new - r_old;
 }
 
 // Likelihood part of one update for one team thread: fetches the expected

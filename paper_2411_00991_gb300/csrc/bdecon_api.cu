@@ -49,7 +49,7 @@ struct ProbHost {
     // arena offsets (bytes)
     size_t o_Ke64 = 0, o_Ke32 = 0;
     size_t o_K64, o_K32, o_dat64, o_dat32, o_ekl, o_wa64, o_m64, o_wa32, o_m32, o_tw64, o_tw32, o_poff;
-    size_t o_sum, o_sq, o_scr, o_samp, o_adapt;
+    size_t o_sum, o_sq, o_scr, o_samp, o_adapt, o_lgam = 0;
     int samp_first = 0;         // first valid kept-object slot (after a resume)
     bool stage_ok = false;      // its chains carry TMA tensor maps for window staging
     bool many = false;          // many independent updates per class step (its team chosen for throughput)
@@ -78,6 +78,9 @@ struct Group {
     int lean_mode = -1;                // lean kernel form: -1 automatic, 0 off, 1 on where eligible
     int user_lean = -2;                // lean_mode set by the autotuner (-2: not set; the handle's setting)
     bool lean = false;                 // the plan runs the lean form
+    bool rows = false;                 // the plan runs the row-run form (bd_rows.cu)
+    int rows_V = 1, rows_VG = 1;       // classes per run, and per team of the block
+    std::vector<CUtensorMap> rmaps;    // its window tensor maps, three per chain in chain order
     int chain_off = 0, n_chains = 0;   // slice of the group-ordered chain table
 };
 
@@ -102,8 +105,9 @@ struct bdecon_handle {
     int lean = -1;                      // lean kernel form: -1 automatic, 0 off, 1 on where eligible
     std::vector<int> prob_group;        // problem -> group
     std::vector<Chain> gch;             // host copy of the group-ordered chain table
-    size_t o_gchains = 0;
+    size_t o_gchains = 0, o_rmaps = 0;
     Chain* d_gchains = nullptr;          // chain descriptors in group order
+    char* d_rmaps = nullptr;             // row-run window maps in group order (kRowMapBytes per chain)
     bool failed = false;
     int sms = 0;
     cudaStream_t st = nullptr;
@@ -305,6 +309,21 @@ int occupancy(int prec, int threads, size_t smem, bool aug, bool fine, int stg, 
     return n;
 }
 
+int occupancy_rows(bool aug, int vg, int threads, size_t smem)
+{
+    static std::mutex mu;
+    static std::map<std::vector<long long>, int> memo;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const std::vector<long long> key = {dev, aug ? 1 : 0, vg, threads, (long long)smem};
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = memo.find(key);
+    if (it != memo.end()) return it->second;
+    const int n = rows_blocks_per_sm(aug, vg, threads, smem);
+    if (n > 0) memo[key] = n;
+    return n;
+}
+
 constexpr size_t kMaxSmem = 227 * 1024;
 
 // One problem's entry in a launch plan: the problem, its update team, its
@@ -362,12 +381,169 @@ bool grow_items(std::vector<PlanItem*>& items)
     return true;
 }
 
+// cuTensorMapEncodeTiled from the driver, looked up once through the runtime
+// (no link-time dependency on the driver library).
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
+{
+    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
+        else
+            cudaGetLastError();
+    });
+    return fn;
+}
+
+// Tensor map of a per-camera-pixel float array of `per` floats a pixel: boxes
+// of bw pixels by L rows, zeros outside the frame.
+bool encode_window_map(const ProbHost& ph, void* base, int per, int bw, CUtensorMap* out)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+    if (!enc) return false;
+    const cuuint32_t es[2] = {1, 1};
+    const cuuint64_t dims[2] = {(cuuint64_t)per * ph.W, (cuuint64_t)ph.H};
+    const cuuint64_t strides[1] = {(cuuint64_t)per * 4 * ph.pitch};
+    const cuuint32_t box[2] = {(cuuint32_t)(per * bw), (cuuint32_t)ph.L};
+    return enc(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Gives the chains of a planned group their tile grids and block ranges.
+void place_items(std::vector<PlanItem*>& items, Group& g)
+{
+    int base = 0;
+    for (PlanItem* it : items) {
+        const int nti = (it->ph->npi + it->tpi - 1) / it->tpi, ntj = (it->ph->npj + it->tpj - 1) / it->tpj;
+        for (Chain* ch : it->chains) {
+            ch->tpi = it->tpi; ch->tpj = it->tpj; ch->nti = nti; ch->ntj = ntj;
+            ch->cta_base = base;
+            base += nti * ntj;
+        }
+    }
+    g.grid = base;
+}
+
+// Plan of the row-run form, where it applies: float problems on the camera
+// grid of one PSF side, stride and team, S >= 3 (a class row of one or two
+// classes has nothing to score together), the run's window box within the TMA
+// limit, and no other form asked for (block warps, streaming, staging, lean).
+//
+// Shape of a block: VG classes scored at once by a team, G teams.
+//  - Small frames of one-warp teams (at most 2 patches per SM) are bound by
+//    the latency of a run: one class per warp, a warp for every class of the
+//    row (64 x 64 frame, L = 9: 0.123 ms a sweep with VG = 3, 0.099 with VG = 1).
+//  - Otherwise VG = 3 with G teams -- or, for teams of four warps (wide
+//    windows, whose blocks shared memory limits before registers do), one team
+//    with VG = 4 or 5 in a 96-register form (1024 x 1024 x 4 chains: L = 31
+//    33.0 ms with VG = 3, 26.7 with 4; L = 25 19.2 and 16.4 with 5) -- whichever
+//    is estimated fastest: an SM's patch-runs (blocks per SM x patches per tile
+//    x runs per row) x teams x (VG + 3, the run's own cost being that of three
+//    classes), at an issue rate that grows with the resident warps W as
+//    W / (W + 16), and 3% a class of the run for scoring again after an
+//    accepted update.  The constants are fitted to sweeps measured at G = 1..4
+//    over L = 9..25, 256 x 256 x 1 to 1024 x 1024 x 4 chains; the estimate
+//    picks the fastest shape or one within 10% of it there.
+bool plan_rows(int precision, int sms, std::vector<PlanItem*>& items, Group& g)
+{
+    g.rows = false;
+    if (precision != BDECON_FP32 || g.fine || g.user_warps || g.streamed || !g.no_stage || g.lean_mode != -1) return false;
+    const PlanItem& i0 = *items[0];
+    const int L = i0.ph->L, S = i0.ph->S, team = i0.team;
+    long long patches = 0;
+    for (const PlanItem* it : items) {
+        if (it->ph->L != L || it->ph->S != S || it->team != team) return false;
+        patches += (long long)it->chains.size() * it->ph->n_patches;
+    }
+    if (S < 3) return false;
+    std::vector<std::pair<int, int>> shapes;   // (VG, G)
+    if (team == 32 && patches <= 2LL * sms) {
+        shapes.push_back({1, std::min(S, 10)});
+    } else {
+        for (int G = 1; G <= std::min(std::max(1, 224 / team), std::min((S + 2) / 3, kRowMaxV / 3)); ++G) shapes.push_back({3, G});
+        if (team == 128) shapes.insert(shapes.end(), {{4, 1}, {5, 1}});
+    }
+    double best = 1e300;
+    std::pair<int, int> best_shape{0, 0};
+    std::vector<std::pair<int, int>> tiles(items.size());
+    for (const auto& shape : shapes) {
+        const int VG = shape.first, G = shape.second;
+        const int V = G * VG, threads = G * team, RN = (S + V - 1) / V;
+        if (4 * rows_box_w(L, V) > 256) continue;
+        for (PlanItem* it : items)
+            if (!it->user) it->tpi = it->tpj = 1;
+        for (;;) {
+            bool one = true;
+            for (const PlanItem* it : items) one = one && it->tpi == 1 && it->tpj == 1;
+            size_t smem = 0;
+            int tot = 0, area = 1;
+            for (const PlanItem* it : items) {
+                smem = std::max(smem, rows_smem(L, S, V, G, team / 32, it->ph->n_tw, it->ph->shape[0].nhalf, g.aug,
+                                                one ? it->ph->max_nhalf : 0).total);
+                tot += item_blocks(*it);
+                area = std::max(area, std::min(it->tpi, it->ph->npi) * std::min(it->tpj, it->ph->npj));
+            }
+            if (smem > kMaxSmem) break;
+            const int bps = occupancy_rows(g.aug, VG, threads, smem);
+            if (bps > 0 && tot <= bps * sms) {
+                const int per_sm = (tot + sms - 1) / sms;
+                const double w = (double)per_sm * threads / 32;
+                const double cost = (double)per_sm * area * RN * G * (VG + 3) * (w + 16.0) / w * (1.0 + 0.03 * V);
+                if (cost < best) {
+                    best = cost;
+                    best_shape = shape;
+                    g.smem = smem;
+                    g.resident = one ? 1 : 0;
+                    for (size_t k = 0; k < items.size(); ++k) tiles[k] = {items[k]->tpi, items[k]->tpj};
+                }
+                break;
+            }
+            if (!grow_items(items)) break;
+        }
+    }
+    if (!best_shape.first) return false;
+    for (size_t k = 0; k < items.size(); ++k) {
+        items[k]->tpi = tiles[k].first;
+        items[k]->tpj = tiles[k].second;
+    }
+    const int VG = best_shape.first, V = best_shape.second * VG, threads = best_shape.second * team;
+    g.rmaps.clear();
+    const int bw = rows_box_w(L, V);
+    for (const PlanItem* it : items)
+        for (const Chain* ch : it->chains) {
+            CUtensorMap m[3];
+            std::memset(m, 0, sizeof m);
+            bool ok = encode_window_map(*it->ph, ch->mu, 1, bw, &m[0]);
+            if (g.aug) ok = ok && encode_window_map(*it->ph, ch->phi, 1, bw, &m[1]);
+            else ok = ok && encode_window_map(*it->ph, ch->cum, 4, bw, &m[1]) && encode_window_map(*it->ph, ch->cum2, 2, bw, &m[2]);
+            if (!ok) return false;
+            g.rmaps.insert(g.rmaps.end(), m, m + 3);
+        }
+    g.threads = threads;
+    g.warps = threads / 32;
+    g.rows_V = V;
+    g.rows_VG = VG;
+    g.stage = 0;
+    g.solo = g.lean = false;
+    g.rows = true;
+    place_items(items, g);
+    return true;
+}
+
 // Launch plan of one group: block = the group's update team (or the user's
 // warps); tiles grow from one patch until every block of every chain of the
 // group is co-resident.  Resident plans (tile state in shared memory) are
 // preferred; if none fits, tile state is streamed from global memory.
 bool plan_items(int precision, int sms, std::vector<PlanItem*>& items, Group& g, std::string& err)
 {
+    if (plan_rows(precision, sms, items, g)) return true;
+    g.rows = false;
+    g.rmaps.clear();
     int team = 32;
     for (const PlanItem* it : items) team = std::max(team, it->team);
     // default block: one update team; two when every problem has many updates
@@ -462,16 +638,7 @@ bool plan_items(int precision, int sms, std::vector<PlanItem*>& items, Group& g,
         if (!(bps > 0 && tot <= bps * sms)) g.solo = false;
     }
     g.lean = want_lean && g.stage == 0 && !g.solo;
-    int base = 0;
-    for (PlanItem* it : items) {
-        const int nti = (it->ph->npi + it->tpi - 1) / it->tpi, ntj = (it->ph->npj + it->tpj - 1) / it->tpj;
-        for (Chain* ch : it->chains) {
-            ch->tpi = it->tpi; ch->tpj = it->tpj; ch->nti = nti; ch->ntj = ntj;
-            ch->cta_base = base;
-            base += nti * ntj;
-        }
-    }
-    g.grid = base;
+    place_items(items, g);
     return true;
 }
 
@@ -520,6 +687,10 @@ bdecon_status make_plan(bdecon_handle* h)
     }
     CK(h, cudaMemcpyAsync(h->d_chains, h->chains.data(), sizeof(Chain) * h->chains.size(), cudaMemcpyHostToDevice, h->st));
     CK(h, cudaMemcpyAsync(h->d_gchains, h->gch.data(), sizeof(Chain) * h->gch.size(), cudaMemcpyHostToDevice, h->st));
+    for (const auto& g : h->groups)
+        if (g.rows)
+            CK(h, cudaMemcpyAsync(h->d_rmaps + (size_t)kRowMapBytes * g.chain_off, g.rmaps.data(),
+                                  sizeof(CUtensorMap) * g.rmaps.size(), cudaMemcpyHostToDevice, h->st));
     return BDECON_OK;
 }
 
@@ -559,44 +730,15 @@ void form_groups(bdecon_handle* h)
     }
 }
 
-// cuTensorMapEncodeTiled from the driver, looked up once through the runtime
-// (no link-time dependency on the driver library).
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
-{
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
-
 // The window-staging tensor maps of one float chain: mu (H x W floats, row
 // pitch mu_pitch), the cumulants c1..c4 (H x 4W floats) and c5, c6 (H x 2W
 // floats); boxes of stage_w(L) pixels by L rows, zeros outside the frame.
 bool encode_stage_maps(const ProbHost& ph, const Chain& ch, CUtensorMap out[3])
 {
-    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (!enc) return false;
-    const cuuint32_t BW = (cuuint32_t)stage_w(ph.L), L = (cuuint32_t)ph.L;
-    const cuuint32_t es[2] = {1, 1};
     void* base[3] = {ch.mu, ch.cum, ch.cum2};
     const int per[3] = {1, 4, 2};   // floats per pixel
-    for (int k = 0; k < 3; ++k) {
-        const cuuint64_t dims[2] = {(cuuint64_t)per[k] * ph.W, (cuuint64_t)ph.H};
-        const cuuint64_t strides[1] = {(cuuint64_t)per[k] * 4 * ph.pitch};
-        const cuuint32_t box[2] = {per[k] * BW, L};
-        if (enc(&out[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base[k], dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return false;
-    }
+    for (int k = 0; k < 3; ++k)
+        if (!encode_window_map(ph, base[k], per[k], stage_w(ph.L), &out[k])) return false;
     return true;
 }
 
@@ -630,6 +772,7 @@ size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainH
         ph.o_samp = ph.p.n_samples > 0 ? A.take(ts * nobj * (size_t)ph.p.n_samples * ph.p.n_chains) : 0;
         const bool adapt = ph.p.adapt_target > 0.0 && ph.p.burn_in > 0;
         ph.o_adapt = adapt ? A.take(16 * (size_t)ph.p.burn_in) : 0;
+        ph.o_lgam = (ph.p.flags & BDECON_FLAG_AUGMENTED) ? A.take(8 * (size_t)kLgamma) : 0;
         const size_t nblk = (npix + kRedThreads - 1) / kRedThreads;
         ph.scr_doubles = std::max(nblk + (size_t)ph.n_patches + 8, nblk + 8 + 2 * (size_t)kMaxS * kMaxS) + 8;
         ph.o_scr = A.take(8 * ph.scr_doubles);
@@ -660,6 +803,7 @@ size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainH
     h->o_imgs = A.take(sizeof(Image) * probs.size());
     h->o_chains = A.take(sizeof(Chain) * chh.size());
     h->o_gchains = A.take(sizeof(Chain) * chh.size());
+    h->o_rmaps = A.take((size_t)kRowMapBytes * chh.size());
     h->o_err = A.take(64);
     h->o_out = A.take(64);
     h->up_bytes = up;
@@ -712,7 +856,19 @@ struct TuneChoice {
     bool staged = false;
     double ms = 1e300;
     bool lean = false;
+    bool rows = false;      // the row-run form (the automatic plan)
 };
+
+// Sets a group up for a tuned choice (before make_plan).
+void apply_choice(Group& g, const TuneChoice& c)
+{
+    g.user_warps = !c.rows;
+    if (!c.rows) g.warps = c.warps;
+    g.streamed = c.streamed;
+    g.no_stage = !c.staged;
+    g.user_stage = true;
+    g.user_lean = c.rows ? -2 : c.lean ? 1 : 0;
+}
 
 // Tuning cache: the autotuner's choices, kept for the life of the process
 // and keyed by the device, the precision, the staging setting and every
@@ -759,14 +915,7 @@ bool apply_cached_plan(bdecon_handle* h)
         form_groups(h);
         return false;
     }
-    for (size_t g = 0; g < h->groups.size(); ++g) {
-        h->groups[g].warps = e.groups[g].warps;
-        h->groups[g].user_warps = true;
-        h->groups[g].streamed = e.groups[g].streamed;
-        h->groups[g].no_stage = !e.groups[g].staged;
-        h->groups[g].user_stage = true;
-        h->groups[g].user_lean = e.groups[g].lean ? 1 : 0;
-    }
+    for (size_t g = 0; g < h->groups.size(); ++g) apply_choice(h->groups[g], e.groups[g]);
     return true;
 }
 
@@ -825,6 +974,7 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
     h->d_imgs = (Image*)(h->arena + h->o_imgs);
     h->d_chains = (Chain*)(h->arena + h->o_chains);
     h->d_gchains = (Chain*)(h->arena + h->o_gchains);
+    h->d_rmaps = h->arena + h->o_rmaps;
     h->d_err = (int*)(h->arena + h->o_err);
     h->d_out = (double*)(h->arena + h->o_out);
     h->d_up = (double*)(h->arena + h->o_up);
@@ -860,6 +1010,8 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
         im.sample_every = ph.p.sample_every > 0 ? ph.p.sample_every : 1;
         im.n_samples = ph.p.n_samples;
         im.adapt_fac = ph.o_adapt ? (const double*)(A + ph.o_adapt) : nullptr;
+        im.lgam = ph.o_lgam ? (const double*)(A + ph.o_lgam) : nullptr;
+        if (im.lgam) launch_lgamma((double*)(A + ph.o_lgam), h->st, &h->launches);
     }
     h->chains.resize(h->chh.size());
     for (int k = 0; k < n; ++k) {
@@ -1000,6 +1152,7 @@ struct LaunchSet {
     std::vector<int> owner;
     const Image* d_imgs = nullptr;
     Chain* d_gch = nullptr;
+    const char* d_rmaps = nullptr;      // row-run window maps in the order of gch
 };
 
 void own_launch_set(bdecon_handle* h, LaunchSet& ls)
@@ -1010,6 +1163,7 @@ void own_launch_set(bdecon_handle* h, LaunchSet& ls)
     ls.owner.assign(h->gch.size(), 0);
     ls.d_imgs = h->d_imgs;
     ls.d_gch = h->d_gchains;
+    ls.d_rmaps = h->d_rmaps;
 }
 
 // Longest segment <= want, starting after sweep t0, that crosses no
@@ -1094,7 +1248,10 @@ bdecon_status run_segment(LaunchSet& ls, int len, cudaStream_t st, bdecon_handle
         a.solo = g.solo ? 1 : 0;
         a.stage = g.stage;
         a.lean = g.lean ? 1 : 0;
-        cudaError_t e = eh->precision == BDECON_FP32 ? launch_sweep<float>(a, g.grid, g.threads, g.smem, st)
+        a.rmaps = g.rows ? ls.d_rmaps + (size_t)kRowMapBytes * g.chain_off : nullptr;
+        a.row_vg = g.rows_VG;
+        cudaError_t e = g.rows ? launch_sweep_rows(a, g.grid, g.threads, g.smem, st)
+                        : eh->precision == BDECON_FP32 ? launch_sweep<float>(a, g.grid, g.threads, g.smem, st)
                                                      : launch_sweep<double>(a, g.grid, g.threads, g.smem, st);
         if (e != cudaSuccess)
             return fail(eh, BDECON_ERR_CUDA, "sweep launch (%d blocks x %d threads, %zu B shared): %s", g.grid,
@@ -1793,6 +1950,22 @@ bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* o
     // already limit the blocks per SM)
     // (the lean form is tried where it applies: float, unstaged)
     const int n_lean = h->precision == BDECON_FP32 ? 2 : 1;
+    // the row-run form first, where some group runs it
+    {
+        for (auto& g : h->groups) apply_choice(g, TuneChoice{0, false, false, 0.0, false, true});
+        bool some = make_plan(h) == BDECON_OK;
+        if (some) {
+            some = false;
+            for (const auto& g : h->groups) some = some || g.rows;
+        }
+        if (some) {
+            std::vector<double> ms;
+            s = tune_trial(h, len, ms);
+            if (s == BDECON_OK) s = restore();
+            for (size_t g = 0; g < ms.size() && s == BDECON_OK; ++g)
+                if (h->groups[g].rows) best[g] = {h->groups[g].warps, false, false, ms[g], false, true};
+        }
+    }
     for (int st = 0; st <= (any_stage ? 1 : 0) && s == BDECON_OK; ++st)
         for (int ln = 0; ln < (st ? 1 : n_lean) && s == BDECON_OK; ++ln)
             for (int streamed = 0; streamed <= 1 && s == BDECON_OK; ++streamed)
@@ -1820,7 +1993,7 @@ bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* o
                     if (s == BDECON_OK) s = restore();
                     for (size_t g = 0; g < ms.size() && s == BDECON_OK; ++g)
                         if (ms[g] < best[g].ms)
-                            best[g] = {h->groups[g].warps, streamed != 0, h->groups[g].stage == 1, ms[g], h->groups[g].lean};
+                            best[g] = {h->groups[g].warps, streamed != 0, h->groups[g].stage == 1, ms[g], h->groups[g].lean, false};
                 }
     double t_groups = 0;
     for (const auto& b : best) t_groups += b.ms;
@@ -1845,7 +2018,7 @@ bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* o
                     std::vector<double> ms;
                     s = tune_trial(h, len, ms);
                     if (s == BDECON_OK) s = restore();
-                    if (s == BDECON_OK && ms[0] < one.ms) one = {w, streamed != 0, g.stage == 1, ms[0], g.lean};
+                    if (s == BDECON_OK && ms[0] < one.ms) one = {w, streamed != 0, g.stage == 1, ms[0], g.lean, false};
                     behind = s == BDECON_OK && one.ms > 1.5 * t_groups;
                 }
     }
@@ -1853,30 +2026,14 @@ bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* o
     if (s == BDECON_OK) {
         h->one_launch = one.ms < t_groups;
         form_groups(h);
-        if (h->one_launch) {
-            h->groups[0].warps = one.warps;
-            h->groups[0].user_warps = true;
-            h->groups[0].streamed = one.streamed;
-            h->groups[0].no_stage = !one.staged;
-            h->groups[0].user_stage = true;
-            h->groups[0].user_lean = one.lean ? 1 : 0;
-        } else {
-            for (size_t g = 0; g < h->groups.size(); ++g) {
-                h->groups[g].warps = best[g].warps;
-                h->groups[g].user_warps = true;
-                h->groups[g].streamed = best[g].streamed;
-                h->groups[g].no_stage = !best[g].staged;
-                h->groups[g].user_stage = true;
-                h->groups[g].user_lean = best[g].lean ? 1 : 0;
-            }
-        }
+        for (size_t g = 0; g < h->groups.size(); ++g) apply_choice(h->groups[g], h->one_launch ? one : best[g]);
         s = make_plan(h);
         if (one_launch) *one_launch = h->one_launch ? 1 : 0;
         if (ms_per_sweep) *ms_per_sweep = (h->one_launch ? one.ms : t_groups) / len;
         if (s == BDECON_OK) {
             TuneEntry e;
             e.one_launch = h->one_launch;
-            for (const auto& g : h->groups) e.groups.push_back({g.warps, g.streamed, g.stage == 1, 0.0, g.lean});
+            for (const auto& g : h->groups) e.groups.push_back({g.warps, g.streamed, g.stage == 1, 0.0, g.lean, g.rows});
             std::lock_guard<std::mutex> lock(g_tune_mu);
             if (g_tune_cache_on) g_tune_cache[tune_key(h)] = e;
         }
@@ -2121,11 +2278,15 @@ bool srv_build(bdecon_server* S, LaunchSet& ls, std::vector<Image>& imgs)
             const Image& im = imgs[ch.img];
             const int n_sub = std::max(1, g.threads / im.team);
             const int rounds = (ch.tpi * ch.tpj + n_sub - 1) / n_sub;
-            S->job_cost[ls.owner[k]] = (int64_t)im.S * im.S * rounds * im.L * im.L;
+            // (row-run form: a block takes its patches one after another, a team VG classes of each at once)
+            S->job_cost[ls.owner[k]] = g.rows ? (int64_t)im.S * ((im.S + g.rows_V - 1) / g.rows_V) * g.rows_VG *
+                                                    ch.tpi * ch.tpj * im.L * im.L
+                                              : (int64_t)im.S * im.S * rounds * im.L * im.L;
         }
     }
     const size_t bi = sizeof(Image) * imgs.size(), bc = sizeof(Chain) * ls.gch.size();
-    if (!srv_tables(S, align_up(bi, 256) + bc + 256)) {
+    const size_t oc = align_up(bi, 256), om = align_up(oc + bc, 256);
+    if (!srv_tables(S, om + (size_t)kRowMapBytes * ls.gch.size() + 256)) {
         S->err = "cudaMalloc of the launch tables failed";
         return false;
     }
@@ -2134,7 +2295,14 @@ bool srv_build(bdecon_server* S, LaunchSet& ls, std::vector<Image>& imgs)
         return false;
     }
     ls.d_imgs = (const Image*)S->d_tab;
-    ls.d_gch = (Chain*)(S->d_tab + align_up(bi, 256));
+    ls.d_gch = (Chain*)(S->d_tab + oc);
+    ls.d_rmaps = S->d_tab + om;
+    for (const Group& g : ls.groups)
+        if (g.rows && cudaMemcpyAsync(S->d_tab + om + (size_t)kRowMapBytes * g.chain_off, g.rmaps.data(),
+                                      sizeof(CUtensorMap) * g.rmaps.size(), cudaMemcpyHostToDevice, S->st) != cudaSuccess) {
+            S->err = "launch table upload failed";
+            return false;
+        }
     return true;
 }
 
