@@ -135,7 +135,9 @@ typedef struct {
 
 /* ------------------------------------------------------------- lifetime */
 
-/* Bytes of device workspace bdecon_create_in needs for these problems.     */
+/* Bytes of device workspace bdecon_create_in needs for these problems.  (In
+ * double 112 bytes a camera pixel and chain of it hold likelihood records
+ * that make the sweep faster; a workspace without them is accepted too.)    */
 bdecon_status bdecon_workspace_size(const bdecon_problem* problems, int32_t n_problems,
                                     size_t* bytes);
 

@@ -10,6 +10,7 @@ namespace bd {
 constexpr int kMaxShapes = 4;       // patch shapes: full, right, bottom, corner
 constexpr int kMaxL = 63;           // largest PSF side
 constexpr int kMaxS = 64;           // largest stride (prior patch side)
+constexpr int kCum64 = 14;           // doubles of a double chain's cumulant record per camera pixel
 constexpr int kMaxSlots = 64;       // sweeps per sweep-kernel launch
 constexpr int kLgamma = 1024;       // photon counts with a tabulated log phi!
 constexpr int kRedThreads = 256;    // fixed block size of every reduction
@@ -72,6 +73,7 @@ struct Chain {
     void* spec;                      // spec_len complex T
     float4* cum;                     // H*mu_pitch photon-posterior cumulants c1..c4 (float chains) or null
     float2* cum2;                    // H*mu_pitch cumulants c5, c6
+    double* cum64;                   // H*mu_pitch records of kCum64 doubles (double marginal chains) or null
     double* rho_sum;                 // Ho*Wo
     double* rho_sq;                  // Ho*Wo or null
     double* trace_part;              // [slot][patch] accepted dL + dP
@@ -182,7 +184,9 @@ __host__ __device__ inline int problem_team(int L, int n_chains, int n_patches, 
 {
     if (team_warps > 0) return 32 * (team_warps > 8 ? 8 : team_warps);
     if ((long long)n_chains * n_patches >= 2048) return !fp32 || L * L <= 128 ? 32 : L * L <= 600 ? 64 : 128;
-    return team_threads(L);
+    // double, few updates per step: four warps from 49 window pixels up, one per
+    // SM sub-partition (each has its own FP64 unit, half a lane a cycle)
+    return fp32 || L * L < 49 ? team_threads(L) : 128;
 }
 
 // Dynamic shared memory of one sweep block: fixed tables, reduction scratch

@@ -263,6 +263,8 @@ __global__ void __launch_bounds__(kRedThreads) k_refresh_mu(Image im, Chain ch, 
             } else {
                 ll = loglik64(mu, d[0], d[1], d[2], d[3]);
             }
+            if (write && ch.cum64)
+                photon_record64(mu, d[0], d[1], d[2], ch.cum64 + kCum64 * ((size_t)a * im.mu_pitch + b));
             if (write && ch.cum) {
                 // the cache describes the stored (rounded) expected image
                 const Cum6 q = photon_cumulants<double>((double)(T)mu, d[0], d[1], d[2]);

@@ -160,6 +160,38 @@ __device__ __forceinline__ void lik_partial(const T* mu_g, const float4* cum_g, 
     }
 }
 
+// Likelihood part of one update for one team thread of a double marginal
+// chain, from the cells' cumulant records (the exact sum beyond their range).
+// Same cells in the same order as lik_partial.
+template <bool RES, bool FINE>
+__device__ __forceinline__ void lik_partial64(const double* mu_g, const double* cum64, const Dat4<double>* dat_s,
+                                              const Dat4<double>* dat_g, const double* Ks, const Image& im, int i, int j,
+                                              int a_lo, int b_lo, int rw, int lt, int NT, double delta, double* out, int lane)
+{
+    const int LL = FINE ? im.Lc * im.Lc : im.L * im.L;
+    double accL = 0;
+    bool badL = false;
+#pragma unroll 2
+    for (int k = lt; k < LL; k += NT) {
+        int aa, bb, kw;
+        if (!win_cell<FINE>(im, i, j, k, aa, bb, kw)) continue;
+        const size_t idx = (size_t)aa * im.mu_pitch + bb;
+        const double xk = mul_rn(delta, Ks[kw]);
+        double y;
+        if (!cgf_delta64(xk, cum64 + kCum64 * idx, y)) {
+            const Dat4<double> dv = RES ? dat_s[(aa - a_lo) * rw + (bb - b_lo)] : dat_g[(size_t)aa * im.W + bb];
+            y = dl_pixel<double>(__ldcg(mu_g + idx), xk, dv.c, dv.is2, dv.beta, badL);
+        }
+        accL += y;
+    }
+    accL = warp_sum(accL);
+    const bool wb = __any_sync(0xffffffffu, badL);
+    if (lane == 0) {
+        out[0] = accL;
+        out[1] = wb ? 1.0 : 0.0;
+    }
+}
+
 // Likelihood part of one update for one team thread from the staged window
 // (float marginal sampler, camera grid): the same cells in the same order
 // with the same arithmetic as lik_partial, the expected image and the
@@ -286,6 +318,8 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
     // float sweeps of the marginal sampler use the cumulant cache; the
     // augmented sampler (AUG) scores windows from the photon counts instead
     constexpr bool CUM = std::is_same<T, float>::value && !AUG;
+    constexpr bool DEC1 = std::is_same<T, double>::value;          // one warp of a team decides
+    constexpr bool C64 = std::is_same<T, double>::value && !AUG;   // cumulant records, where the chain has them
     static_assert(STG == 0 || (std::is_same<T, float>::value && !AUG && !FINE && !SOLO), "staging: float marginal camera grid");
     constexpr bool SANY = STG != 0;                          // staging
     constexpr bool SWIN = STG == 1;                          // the window is staged
@@ -298,6 +332,7 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
     __shared__ int s_stale;
     __shared__ int s_acc_any;
     __shared__ int s_pub;
+    __shared__ int s_dec[8];   // a team's decision, as its first warp took it (double)
     __shared__ int s_chg;   // the last published step changed data (thread 0 only)
     __shared__ int s_word;  // the last published progress word (thread 0 only)
     __shared__ double s_phid[AUG ? 8 : 1][8];   // photon-count step: [sub-team][warp] log-density changes
@@ -734,7 +769,7 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
             // latency overlaps the arithmetic below
             if (active && !SWIN) {
                 if constexpr (AUG) window_fetch_aug<T, FINE, NPX>(mu_g, phi_g, im, i, j, muv, phv, lt);
-                else window_fetch<T, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, im, i, j, lt, muv, cq, cq2, lt);
+                else if (!C64 || ch.cum64 == nullptr) window_fetch<T, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, im, i, j, lt, muv, cq, cq2, lt);
             }
             // a2 + a4: proposal and prior change (own tile state only)
             if (active) {
@@ -779,9 +814,19 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
                 else if constexpr (SWIN)
                     lik_partial_staged<RES>(wmu, wcum, wcum2, BW, wdx, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt,
                                             NT, delta, pr2 + twarp * 4, lane);
-                else
-                    lik_partial<T, RES, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT,
-                                             delta, muv, pr2 + twarp * 4, lane, cq, cq2, true);
+                else {
+                    bool done = false;
+                    if constexpr (C64) {
+                        if (ch.cum64 != nullptr) {
+                            lik_partial64<RES, FINE>(mu_g, ch.cum64, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT, delta,
+                                                     pr2 + twarp * 4, lane);
+                            done = true;
+                        }
+                    }
+                    if (!done)
+                        lik_partial<T, RES, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt,
+                                                            NT, delta, muv, pr2 + twarp * 4, lane, cq, cq2, true);
+                }
             }
             // a5: Metropolis-Hastings decision with the Hastings term of the log-space
             // walk, taken from the round's partial sums as soon as every warp of the
@@ -811,7 +856,18 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
                 nonfin = !bad && !(fabs(tot) <= (T)P::kMaxFinite);
                 accept = !bad && !nonfin && (lu < tot + z);   // z holds s_m z
             };
-            if (active) decide();
+            // (double: the team's first warp alone -- the division and logarithm cost
+            // a sub-partition's FP64 unit as much for a uniform operand)
+            if (active) {
+                if constexpr (DEC1) {
+                    if (twarp == 0) {
+                        decide();
+                        if (lane == 0) s_dec[g] = accept ? 1 : 0;
+                    }
+                } else {
+                    decide();
+                }
+            }
             // the next step's draw, after the step barrier so that the other warps
             // need not wait for it there; it overlaps the neighbour wait below
             if (ahead && in_team && twarp == pwarp) {
@@ -857,7 +913,16 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
             // barrier does; team barriers: a team's decision is uniform in it)
             const bool blk = r == 0 || !tb;
             int any_accept;
-            if constexpr (SOLO) {
+            if constexpr (DEC1) {
+                if (blk) {
+                    any_accept = __syncthreads_or(active && twarp == 0 && accept ? 1 : 0);
+                    accept = active && s_dec[g] != 0;
+                } else {
+                    tsync();
+                    accept = active && s_dec[g] != 0;
+                    any_accept = accept ? 1 : 0;
+                }
+            } else if constexpr (SOLO) {
                 __syncthreads();
                 any_accept = active && accept ? 1 : 0;
             } else if (blk) {
@@ -888,8 +953,17 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
                         lik_partial_staged<RES>(wmu, wcum, wcum2, BW, wdx, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw,
                                                 lt, NT, delta, pr2 + twarp * 4, lane);
                     } else {
-                        lik_partial<T, RES, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT,
-                                                 delta, muv, pr2 + twarp * 4, lane, cq, cq2, false);
+                        bool done = false;
+                        if constexpr (C64) {
+                            if (ch.cum64 != nullptr) {
+                                lik_partial64<RES, FINE>(mu_g, ch.cum64, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT,
+                                                         delta, pr2 + twarp * 4, lane);
+                                done = true;
+                            }
+                        }
+                        if (!done)
+                            lik_partial<T, RES, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw,
+                                                                lt, NT, delta, muv, pr2 + twarp * 4, lane, cq, cq2, false);
                     }
                 }
                 __syncthreads();
@@ -916,10 +990,20 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
                                 // (unchanged since)
                                 const size_t idx = (size_t)aa * im.mu_pitch + bb;
                                 const int widx = (k / L) * BW + wdx + (k - (k / L) * L);
-                                const T old = SWIN ? (T)wmu[widx] : one_batch ? muv[jj] : __ldcg(mu_g + idx);
+                                const T old = SWIN ? (T)wmu[widx] : one_batch && !(C64 && ch.cum64 != nullptr) ? muv[jj] : __ldcg(mu_g + idx);
                                 const T xk = mul_rn(delta, Ks[kw]);
                                 const T nmu = add_rn(old, xk);
                                 __stcg(mu_g + idx, nmu);
+                                if constexpr (C64) {
+                                    if (ch.cum64 != nullptr) {
+                                        double* rec = ch.cum64 + kCum64 * idx;
+                                        if (!cum64_shift(nmu, xk, rec)) {
+                                            const Dat4<T> dv =
+                                                RES ? dat_s[(aa - a_lo) * rw + (bb - b_lo)] : dat_g[(size_t)aa * W + bb];
+                                            photon_record64(nmu, dv.c, dv.is2, dv.beta, rec);
+                                        }
+                                    }
+                                }
                                 if (CUM) {
                                     const float d = (float)xk * Prec<float>::rcp((float)old);
                                     Cum6 nq;
@@ -1179,6 +1263,13 @@ __global__ void __launch_bounds__(256) k_delta(const Image* imp, const Chain* ch
                     const float d = (float)xk * Prec<float>::rcp((float)mu[idx]);
                     if (fabsf(d) <= kCumEval) {
                         accL += (T)cgf_delta((float)xk, log1p_cum(d), ch.cum[idx], ch.cum2[idx]);
+                        continue;
+                    }
+                }
+                if constexpr (std::is_same<T, double>::value) {
+                    double y;
+                    if (ch.cum64 != nullptr && cgf_delta64(xk, ch.cum64 + kCum64 * idx, y)) {
+                        accL += y;
                         continue;
                     }
                 }

@@ -85,7 +85,7 @@ struct Group {
 };
 
 struct ChainHost {
-    size_t o_rho, o_mu, o_spec, o_cum, o_cum2, o_tpart, o_acc, o_log, o_prog, o_trace, o_tdev, o_steps, o_phi;
+    size_t o_rho, o_mu, o_spec, o_cum, o_cum2, o_cum64, o_tpart, o_acc, o_log, o_prog, o_trace, o_tdev, o_steps, o_phi;
     size_t o_tmap = 0;
 };
 
@@ -539,9 +539,8 @@ bool plan_rows(int precision, int sms, std::vector<PlanItem*>& items, Group& g)
 // warps); tiles grow from one patch until every block of every chain of the
 // group is co-resident.  Resident plans (tile state in shared memory) are
 // preferred; if none fits, tile state is streamed from global memory.
-bool plan_items(int precision, int sms, std::vector<PlanItem*>& items, Group& g, std::string& err)
+bool plan_general(int precision, int sms, std::vector<PlanItem*>& items, Group& g, std::string& err)
 {
-    if (plan_rows(precision, sms, items, g)) return true;
     g.rows = false;
     g.rmaps.clear();
     int team = 32;
@@ -640,6 +639,38 @@ bool plan_items(int precision, int sms, std::vector<PlanItem*>& items, Group& g,
     g.lean = want_lean && g.stage == 0 && !g.solo;
     place_items(items, g);
     return true;
+}
+
+// The row-run form where it applies, else the general forms.  In double,
+// resident tile state can leave so little shared memory that few warps are
+// resident; the streamed plan is taken where the estimate of plan_rows (tile
+// patches per SM at an issue rate growing with the resident warps) puts it at
+// least 10% ahead (300 x 300 L = 9 x 4 chains 25.1 -> 18.9 ms a sweep,
+// 512 x 512 L = 17 50 -> 34).
+bool plan_items(int precision, int sms, std::vector<PlanItem*>& items, Group& g, std::string& err)
+{
+    if (plan_rows(precision, sms, items, g)) return true;
+    if (precision == BDECON_FP64 && !g.streamed && g.no_stage) {
+        auto cost = [&](const Group& q) {
+            int area = 1;
+            for (const PlanItem* it : items)
+                area = std::max(area, std::min(it->tpi, it->ph->npi) * std::min(it->tpj, it->ph->npj));
+            const int per_sm = (q.grid + sms - 1) / sms;
+            const double w = (double)per_sm * q.warps;
+            return (double)per_sm * area * (w + 16.0) / w;
+        };
+        const bool ok = plan_general(precision, sms, items, g, err);
+        const double c = ok ? cost(g) : 1e300;
+        Group st = g;
+        st.streamed = true;
+        std::string err2;
+        if (plan_general(precision, sms, items, st, err2) && cost(st) < 0.9 * c) {
+            st.streamed = false;   // (the caller's setting)
+            g = st;
+            return true;
+        }
+    }
+    return plan_general(precision, sms, items, g, err);
 }
 
 void drop_graphs(bdecon_handle* h)
@@ -742,7 +773,11 @@ bool encode_stage_maps(const ProbHost& ph, const Chain& ch, CUtensorMap out[3])
     return true;
 }
 
-size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainHost>& chh, int prec, int max_sweeps)
+// Device arena layout.  records: with the double chains' cumulant records
+// (112 bytes a camera pixel); without them the double sweep evaluates the
+// exact photon sums, and the arena is the smallest that works.
+size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainHost>& chh, int prec, int max_sweeps,
+              bool records = true)
 {
     Alloc A;
     const size_t ts = prec == BDECON_FP32 ? 4 : 8;
@@ -787,6 +822,7 @@ size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainH
             const bool aug = (ph.p.flags & BDECON_FLAG_AUGMENTED) != 0;
             x.o_cum = prec == BDECON_FP32 && !aug ? A.take(16 * (size_t)ph.H * ph.pitch) : 0;
             x.o_cum2 = prec == BDECON_FP32 && !aug ? A.take(8 * (size_t)ph.H * ph.pitch) : 0;
+            x.o_cum64 = prec == BDECON_FP64 && !aug && records ? A.take(8 * (size_t)kCum64 * ph.H * ph.pitch) : 0;
             x.o_phi = aug ? A.take(ts * (size_t)ph.H * ph.pitch) : 0;
             x.o_tpart = A.take(8 * (size_t)kMaxSlots * ph.n_patches);
             x.o_acc = A.take(8 * (size_t)max_sweeps);
@@ -919,7 +955,8 @@ bool apply_cached_plan(bdecon_handle* h)
     return true;
 }
 
-bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* ws, size_t ws_bytes, bdecon_handle** out)
+bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* ws, size_t ws_bytes, bdecon_handle** out,
+                          bool records = true)
 {
     if (!out) return fail(nullptr, BDECON_ERR_INVALID, "out is NULL");
     *out = nullptr;
@@ -954,15 +991,23 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (!coop) return bail(fail(h, BDECON_ERR_CUDA, "device does not support cooperative launches"));
-    const size_t need = layout(h, h->probs, h->chh, h->precision, h->max_sweeps);
+    // (the cumulant records of double chains are left out where memory is short)
+    size_t need = layout(h, h->probs, h->chh, h->precision, h->max_sweeps, records);
     if (ws) {
+        if (ws_bytes < need && records) need = layout(h, h->probs, h->chh, h->precision, h->max_sweeps, false);
         if (ws_bytes < need) return bail(fail(h, BDECON_ERR_NOMEM, "workspace of %zu bytes, %zu needed", ws_bytes, need));
         if (((uintptr_t)ws) % 256) return bail(fail(h, BDECON_ERR_INVALID, "workspace must be 256-byte aligned"));
         h->arena = (char*)ws;
         h->own_arena = false;
     } else {
         void* p = nullptr;
-        if (cudaMalloc(&p, need) != cudaSuccess) {
+        cudaError_t e = cudaMalloc(&p, need);
+        if (e != cudaSuccess && records && h->precision == BDECON_FP64) {
+            cudaGetLastError();
+            need = layout(h, h->probs, h->chh, h->precision, h->max_sweeps, false);
+            e = cudaMalloc(&p, need);
+        }
+        if (e != cudaSuccess) {
             cudaGetLastError();
             return bail(fail(h, BDECON_ERR_NOMEM, "cudaMalloc of %zu bytes failed", need));
         }
@@ -1026,6 +1071,7 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
             ch.rho = A + x.o_rho; ch.mu = A + x.o_mu; ch.spec = A + x.o_spec;
             ch.cum = x.o_cum ? (float4*)(A + x.o_cum) : nullptr;
             ch.cum2 = x.o_cum2 ? (float2*)(A + x.o_cum2) : nullptr;
+            ch.cum64 = x.o_cum64 ? (double*)(A + x.o_cum64) : nullptr;
             ch.rho_sum = (double*)(A + ph.o_sum) + c * nobj;
             ch.rho_sq = ph.o_sq ? (double*)(A + ph.o_sq) + c * nobj : nullptr;
             ch.trace_part = (double*)(A + x.o_tpart);
@@ -1374,7 +1420,7 @@ bdecon_status chain_index(bdecon_handle* h, int p, int c, int* ci)
 
 extern "C" {
 
-bdecon_status bdecon_workspace_size(const bdecon_problem* ps, int32_t n, size_t* bytes)
+static bdecon_status workspace_size(const bdecon_problem* ps, int32_t n, size_t* bytes, bool records)
 {
     if (!ps || n < 1 || !bytes) return fail(nullptr, BDECON_ERR_INVALID, "bad arguments");
     for (int k = 0; k < n; ++k) {
@@ -1390,8 +1436,13 @@ bdecon_status bdecon_workspace_size(const bdecon_problem* ps, int32_t n, size_t*
         ms = std::max(ms, ps[k].max_sweeps ? ps[k].max_sweeps : 4096);
     }
     std::vector<ChainHost> chh;
-    *bytes = layout(&tmp, probs, chh, ps[0].precision, ms);
+    *bytes = layout(&tmp, probs, chh, ps[0].precision, ms, records);
     return BDECON_OK;
+}
+
+bdecon_status bdecon_workspace_size(const bdecon_problem* ps, int32_t n, size_t* bytes)
+{
+    return workspace_size(ps, n, bytes, true);
 }
 
 bdecon_status bdecon_create(const bdecon_problem* p, void* stream, bdecon_handle** out)
@@ -2133,6 +2184,7 @@ struct SrvJob {
     int state = BDECON_JOB_QUEUED;
     double t_submit = 0, t_start = 0, t_done = 0;
     size_t mem = 0;
+    bool records = true;                // with the double chains' cumulant records (where the budget holds them)
     bdecon_handle* h = nullptr;
     std::vector<double> mean;
     std::string err;
@@ -2342,7 +2394,7 @@ void srv_loop(bdecon_server* S)
             }
         }
         for (SrvJob* j : admit) {
-            bdecon_status st = bdecon_create(&j->p, S->st, &j->h);
+            bdecon_status st = create_impl(&j->p, 1, S->st, nullptr, 0, &j->h, j->records);
             if (st != BDECON_OK) {
                 j->h = nullptr;
                 srv_finish(S, j, BDECON_JOB_FAILED, bdecon_last_error(nullptr));
@@ -2481,7 +2533,11 @@ bdecon_status bdecon_server_submit(bdecon_server* S, const bdecon_problem* p, in
     j->p.flags = p->flags & BDECON_FLAG_AUGMENTED;
     j->sweeps = j->remaining = sweeps;
     size_t bytes = 0;
-    st = bdecon_workspace_size(&j->p, 1, &bytes);
+    st = workspace_size(&j->p, 1, &bytes, true);
+    if (st == BDECON_OK && bytes > S->cfg.mem_budget) {
+        j->records = false;
+        st = workspace_size(&j->p, 1, &bytes, false);
+    }
     if (st != BDECON_OK) {
         delete j;
         return st;
