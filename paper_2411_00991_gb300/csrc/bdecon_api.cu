@@ -1637,7 +1637,7 @@ bdecon_status bdecon_posterior_quantiles(bdecon_handle* h, int32_t p, const doub
         for (int k = 0; k < nq; ++k)
             CK(h, cudaMemcpyAsync(out + (size_t)k * npix + p0, dout + (size_t)k * np, 8 * (size_t)np,
                                   cudaMemcpyDeviceToHost, h->st));
-        CK(h, cudaStreamSynchronize(h->st));   // the staging buffer is reused by the next chunk
+        // (the staging buffer is reused by the next chunk, in stream order)
     }
     return check_device(h);
 }
