@@ -62,7 +62,7 @@ struct Image {
     const float* Ke32;
     int sample_every, n_samples;     // kept objects: every sample_every-th sweep past burn-in, n_samples slots
     const double* adapt_fac;         // [burn_in][2] proposal-scale factors after accept / reject, or null
-    const double* lgam;              // log phi! of the first kLgamma photon counts (augmented problems), or null
+    const double* lgam;              // log phi! of the first kLgamma photon counts
 };
 
 // One chain (an instance of a problem with its own state and random stream).
@@ -279,6 +279,15 @@ __host__ __device__ inline RowsSmem rows_smem(int L, int S, int V, int G, int nw
     p.spec = o; o += al16((size_t)spec_entries * 8);
     p.total = o;
     return p;
+}
+
+// Blocks of the expected-image refresh: tiles of 32 x 4 camera pixels while
+// those leave SMs free, else of 64 x 16; a finer lattice takes 256 pixels a block.
+inline bool refresh_small(int H, int W) { return (int64_t)H * W <= 256 * 1024; }
+inline int refresh_blocks(int H, int W, int f)
+{
+    if (f > 1) return (H * W + kRedThreads - 1) / kRedThreads;
+    return refresh_small(H, W) ? ((W + 31) / 32) * ((H + 3) / 4) : ((W + 63) / 64) * ((H + 15) / 16);
 }
 
 // host launchers (defined in the .cu files)

@@ -124,39 +124,55 @@ __global__ void k_setup_tw(int n, double* tw64, float* tw32)
 // Eq. 8 hyperparameter for one patch shape: alpha = |DFT(PSF wrapped onto the
 // ph x pw torus, centre at the origin)| / sum, then the weights of the
 // canonical half-spectrum entries: mult * (alpha - 1) / 2 and mult.
+//
+// One block: the wrapped kernel gathered per torus pixel, its transform taken
+// by rows and then columns in shared memory (ph pw (ph + pw) products; the
+// direct sum and a one-thread wrap took 646 us at 25 x 25, four shapes a problem).
 __global__ void __launch_bounds__(kRedThreads) k_setup_alpha(int L, const double* K64, int ph, int pw,
-                                                            const int* ent_kl, int nhalf, double* kw,
-                                                            double* mag, double* wa64, double* m64,
-                                                            float* wa32, float* m32, const double2* twh,
+                                                            const int* ent_kl, int nhalf, double* mag, double* wa64,
+                                                            double* m64, float* wa32, float* m32, const double2* twh,
                                                             const double2* tww)
 {
+    extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ double sh[kRedThreads];
     const int R = L / 2, n = ph * pw;
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < n; ++k) kw[k] = 0.0;
-        for (int p = 0; p < L; ++p)
-            for (int q = 0; q < L; ++q) {
-                const int x = ((p - R) % ph + ph) % ph, y = ((q - R) % pw + pw) % pw;
-                kw[x * pw + y] += K64[p * L + q];
-            }
+    double2* Y = reinterpret_cast<double2*>(dyn);           // [ph][pw]
+    double* x = reinterpret_cast<double*>(Y + n);           // [ph][pw]
+    for (int e = threadIdx.x; e < n; e += kRedThreads) {
+        // kernel rows p with (p - R) mod ph = u, columns alike
+        const int u = e / pw, v = e - u * pw;
+        double k = 0.0;
+        for (int p = (u + R) % ph; p < L; p += ph)
+            for (int q = (v + R) % pw; q < L; q += pw) k += K64[p * L + q];
+        x[e] = k;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < n; e += kRedThreads) {
+        const int u = e / pw, l = e - u * pw;
+        double re = 0.0, im = 0.0;
+        for (int v = 0, j = 0; v < pw; ++v) {
+            const double2 w = tww[j];
+            re += x[u * pw + v] * w.x;
+            im += x[u * pw + v] * w.y;
+            j += l;
+            j -= j >= pw ? pw : 0;
+        }
+        Y[e] = make_double2(re, im);
     }
     __syncthreads();
     double part = 0.0;
-    for (int idx = threadIdx.x; idx < n; idx += kRedThreads) {
-        const int k = idx / pw, l = idx % pw;
-        // exp(-2 pi i (k u / ph + l v / pw)) from the twiddle tables of the two sides
+    for (int e = threadIdx.x; e < n; e += kRedThreads) {
+        const int k = e / pw, l = e - k * pw;
         double re = 0.0, im = 0.0;
-        for (int u = 0; u < ph; ++u) {
-            const double2 eh = twh[(k * u) % ph];
-            for (int v = 0; v < pw; ++v) {
-                const double2 ew = tww[(l * v) % pw];
-                const double x = kw[u * pw + v];
-                re += x * (eh.x * ew.x - eh.y * ew.y);
-                im += x * (eh.x * ew.y + eh.y * ew.x);
-            }
+        for (int u = 0, j = 0; u < ph; ++u) {
+            const double2 w = twh[j], y = Y[u * pw + l];
+            re += y.x * w.x - y.y * w.y;
+            im += y.x * w.y + y.y * w.x;
+            j += k;
+            j -= j >= ph ? ph : 0;
         }
-        mag[idx] = hypot(re, im);
-        part += mag[idx];
+        mag[e] = hypot(re, im);
+        part += mag[e];
     }
     // the sum over all frequencies, in a fixed order
     __syncthreads();
@@ -211,10 +227,18 @@ void launch_setup(const Image& im, const Image* d_im, const float* w, const floa
                                       const_cast<float*>(im.tw32) + 2 * sh.twh_off);
         k_setup_tw<<<1, 128, 0, st>>>(sh.pw, const_cast<double*>(im.tw64) + 2 * sh.tww_off,
                                       const_cast<float*>(im.tw32) + 2 * sh.tww_off);
-        double* kw = scratch + nblk + 8;
-        double* mag = kw + kMaxS * kMaxS;
-        k_setup_alpha<<<1, kRedThreads, 0, st>>>(im.L, im.K64, sh.ph, sh.pw, im.ent_kl + sh.ent_off, sh.nhalf, kw,
-                                                 mag, const_cast<double*>(im.ent_wa64) + sh.ent_off,
+        double* mag = scratch + nblk + 8;
+        const size_t sm = 24 * (size_t)sh.ph * sh.pw;
+        static std::atomic<size_t> limit{46 * 1024};   // the dynamic shared-memory limit only grows (the static sums count too)
+        static std::mutex mu;
+        if (sm > limit.load()) {
+            std::lock_guard<std::mutex> lock(mu);
+            if (sm > limit.load() &&
+                cudaFuncSetAttribute(k_setup_alpha, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess)
+                limit.store(sm);
+        }
+        k_setup_alpha<<<1, kRedThreads, sm, st>>>(im.L, im.K64, sh.ph, sh.pw, im.ent_kl + sh.ent_off, sh.nhalf, mag,
+                                                 const_cast<double*>(im.ent_wa64) + sh.ent_off,
                                                  const_cast<double*>(im.ent_m64) + sh.ent_off,
                                                  const_cast<float*>(im.ent_wa32) + sh.ent_off,
                                                  const_cast<float*>(im.ent_m32) + sh.ent_off,
@@ -236,9 +260,99 @@ template void launch_init_rho<double>(const Image&, const Chain&, const double*,
 
 // ------------------------------------------------------------------ a8 ---
 // mu = K (x) rho (Eq. 1-2) and the per-pixel log likelihood (Eq. 6), double.
+// A block takes a tile of TW x (TY RJ) camera pixels, its object values
+// converted to double once into shared memory (read straight from the float
+// object, each product paid a conversion, on the FP64 unit as well).  A thread
+// sums RJ pixels TY rows apart, so a kernel entry is loaded once for RJ
+// products.  Bound by the FP64 unit (half a lane a cycle per sub-partition):
+// L^2 products and about 170..290 operations of the photon sum a pixel; 1024 x
+// 1024, L = 25, with the cumulants: 4.2 -> 2.1 ms.  Small frames take 128-pixel
+// tiles, one pixel a thread, to reach more SMs.
+__device__ __forceinline__ double block_sum_n(double v, double* sh, int n)
+{
+    const int tid = threadIdx.x;
+    sh[tid] = v;
+    __syncthreads();
+    for (int o = n / 2; o > 0; o >>= 1) {
+        if (tid < o) sh[tid] += sh[tid + o];
+        __syncthreads();
+    }
+    return sh[0];
+}
+
+// log likelihood of camera pixel (a, b) at mu; with write, the state derived from mu
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_refresh_mu(Image im, Chain ch, double* part_ll, int write,
-                                                           int* err)
+__device__ __forceinline__ double refresh_pixel(const Image& im, const Chain& ch, int a, int b, double mu, int write, int* err)
+{
+    const size_t x = (size_t)a * im.mu_pitch + b;
+    double ll = 0.0;
+    if (!(mu > 0.0) || !isfinite(mu)) {
+        atomicOr(err, kErrNumeric);
+    } else {
+        const double* d = im.dat64 + 4 * ((size_t)a * im.W + b);
+        Cum6 q;
+        if (write && ch.phi) {   // augmented chain: the completed likelihood at its counts
+            const int phi = (int)reinterpret_cast<const T*>(ch.phi)[x];
+            ll = d[3] + phi_logterm_tab(phi, ::log((double)(T)mu), d[0], d[1], im.lgam) - (double)(T)mu;
+        } else if (write && ch.cum) {
+            // the cache describes the stored (rounded) expected image
+            ll = loglik_sum64<true>(mu, (double)(T)mu, d[0], d[1], d[2], d[3], im.lgam, q);
+            ch.cum[x] = q.a;
+            ch.cum2[x] = q.b;
+        } else if (write && ch.cum64) {
+            const double S = photon_record64(mu, d[0], d[1], d[2], ch.cum64 + kCum64 * x);
+            ll = loglik_from_sum64(mu, d[0], d[1], d[3], S, photon_mode((float)mu, (float)d[0], (float)d[1]), im.lgam);
+        } else {
+            ll = loglik_sum64<false>(mu, mu, d[0], d[1], d[2], d[3], im.lgam, q);
+        }
+    }
+    if (write) reinterpret_cast<T*>(ch.mu)[x] = (T)mu;
+    return ll;
+}
+
+template <typename T, int TW, int TY, int RJ>
+__global__ void __launch_bounds__(TW * TY) k_refresh_mu(Image im, Chain ch, double* part_ll, int write, int* err)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ double sh[TW * TY];
+    const int L = im.L, tid = threadIdx.x, TC = TW + L - 1, TR = TY * RJ + L - 1;
+    double* K = reinterpret_cast<double*>(dyn);                 // [L][L]
+    double* r = K + ((L * L + 1) & ~1);                         // [TR][TC]
+    const int ntw = (im.W + TW - 1) / TW;
+    const int a0 = blockIdx.x / ntw * (TY * RJ), b0 = blockIdx.x % ntw * TW;
+    const T* rho = reinterpret_cast<const T*>(ch.rho);
+    for (int k = tid; k < L * L; k += TW * TY) K[k] = im.Ke64[k];
+    for (int k = tid; k < TR * TC; k += TW * TY) {
+        const int i = a0 + k / TC, j = b0 + k % TC;
+        r[k] = i < im.Ho && j < im.Wo ? (double)rho[(size_t)i * im.Wo + j] : 0.0;
+    }
+    __syncthreads();
+    // mu[a][b] = sum K[p][q] rho[a + L-1-p][b + L-1-q]
+    const int tx = tid % TW, ty = tid / TW;
+    double mu[RJ];
+#pragma unroll
+    for (int j = 0; j < RJ; ++j) mu[j] = 0.0;
+    for (int p = 0; p < L; ++p) {
+        const double* row = r + (ty + L - 1 - p) * TC + tx + L - 1;
+        for (int q = 0; q < L; ++q) {
+            const double k = K[p * L + q];
+#pragma unroll
+            for (int j = 0; j < RJ; ++j) mu[j] += k * row[j * TY * TC - q];
+        }
+    }
+    double ll = 0.0;
+#pragma unroll
+    for (int j = 0; j < RJ; ++j) {
+        const int a = a0 + ty + j * TY, b = b0 + tx;
+        if (a < im.H && b < im.W) ll += refresh_pixel<T>(im, ch, a, b, mu[j], write, err);
+    }
+    const double s = block_sum_n(ll, sh, TW * TY);
+    if (tid == 0) part_ll[blockIdx.x] = s;
+}
+
+// Object lattice finer than the camera: straight from the object.
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads) k_refresh_mu_fine(Image im, Chain ch, double* part_ll, int write, int* err)
 {
     __shared__ double sh[kRedThreads];
     const int idx = blockIdx.x * kRedThreads + threadIdx.x;
@@ -253,26 +367,7 @@ __global__ void __launch_bounds__(kRedThreads) k_refresh_mu(Image im, Chain ch, 
             const T* row = rho + (size_t)(f * a + Le - 1 - p) * im.Wo + (f * b + Le - 1);
             for (int q = 0; q < Le; ++q) mu += im.Ke64[p * Le + q] * (double)row[-q];
         }
-        if (!(mu > 0.0) || !isfinite(mu)) {
-            atomicOr(err, kErrNumeric);
-        } else {
-            const double* d = im.dat64 + 4 * (size_t)idx;
-            if (write && ch.phi) {   // augmented chain: the completed likelihood at its counts
-                const int phi = (int)reinterpret_cast<const T*>(ch.phi)[(size_t)a * im.mu_pitch + b];
-                ll = d[3] + phi_logterm(phi, ::log((double)(T)mu), d[0], d[1]) - (double)(T)mu;
-            } else {
-                ll = loglik64(mu, d[0], d[1], d[2], d[3]);
-            }
-            if (write && ch.cum64)
-                photon_record64(mu, d[0], d[1], d[2], ch.cum64 + kCum64 * ((size_t)a * im.mu_pitch + b));
-            if (write && ch.cum) {
-                // the cache describes the stored (rounded) expected image
-                const Cum6 q = photon_cumulants<double>((double)(T)mu, d[0], d[1], d[2]);
-                ch.cum[(size_t)a * im.mu_pitch + b] = q.a;
-                ch.cum2[(size_t)a * im.mu_pitch + b] = q.b;
-            }
-        }
-        if (write) reinterpret_cast<T*>(ch.mu)[(size_t)a * im.mu_pitch + b] = (T)mu;
+        ll = refresh_pixel<T>(im, ch, a, b, mu, write, err);
     }
     const double s = block_sum(ll, sh);
     if (threadIdx.x == 0) part_ll[blockIdx.x] = s;
@@ -304,13 +399,17 @@ __global__ void __launch_bounds__(kRedThreads) k_refresh_spec(Image im, Chain ch
         x[e] = (double)rho[(size_t)u * im.Wo + v];
     }
     __syncthreads();
+    // (every l, although the rows are real: the table's conjugate twiddles differ
+    // in their last place, which would turn float roundings of small coefficients)
     for (int e = threadIdx.x; e < n; e += kRedThreads) {
-        const int u = e / pw, l = e - (e / pw) * pw;
+        const int u = e / pw, l = e - u * pw;
         double re = 0.0, imv = 0.0;
-        for (int v = 0; v < pw; ++v) {
-            const double2 w = tww[(l * v) % pw];
+        for (int v = 0, j = 0; v < pw; ++v) {
+            const double2 w = tww[j];
             re += x[u * pw + v] * w.x;
             imv += x[u * pw + v] * w.y;
+            j += l;
+            j -= j >= pw ? pw : 0;
         }
         Y[e] = make_double2(re, imv);
     }
@@ -322,11 +421,13 @@ __global__ void __launch_bounds__(kRedThreads) k_refresh_spec(Image im, Chain ch
         const int kl = im.ent_kl[sp.ent_off + e];
         const int k = kl >> 16, l = kl & 0xffff;
         double re = 0.0, imv = 0.0;
-        for (int u = 0; u < ph; ++u) {
-            const double2 w = twh[(k * u) % ph];
+        for (int u = 0, j = 0; u < ph; ++u) {
+            const double2 w = twh[j];
             const double2 y = Y[u * pw + l];
             re += y.x * w.x - y.y * w.y;
             imv += y.x * w.y + y.y * w.x;
+            j += k;
+            j -= j >= ph ? ph : 0;
         }
         if (write) {
             T2 X;
@@ -359,10 +460,27 @@ template <typename T>
 void launch_refresh(const Image& im, const Chain& ch, double* scratch, int write_state, double* out_logpost,
                     const int* out_index, int* err, cudaStream_t st, int64_t* launches)
 {
-    const int nblk = (im.H * im.W + kRedThreads - 1) / kRedThreads;
+    const int nblk = refresh_blocks(im.H, im.W, im.f);
     double* part_ll = scratch;
     double* part_lp = scratch + nblk;
-    k_refresh_mu<T><<<nblk, kRedThreads, 0, st>>>(im, ch, part_ll, write_state, err);
+    if (im.f > 1) {
+        k_refresh_mu_fine<T><<<nblk, kRedThreads, 0, st>>>(im, ch, part_ll, write_state, err);
+    } else {
+        const bool small = refresh_small(im.H, im.W);
+        const void* fn = small ? (const void*)k_refresh_mu<T, 32, 4, 1> : (const void*)k_refresh_mu<T, 64, 4, 4>;
+        const int TC = (small ? 32 : 64) + im.L - 1, TR = (small ? 4 : 16) + im.L - 1;
+        const size_t sm = 8 * (size_t)(((im.L * im.L + 1) & ~1) + TC * TR);
+        static std::atomic<size_t> lim[2] = {{48 * 1024 - 2048}, {48 * 1024 - 2048}};   // (the static sums count too)
+        static std::mutex mu_lim;
+        if (sm > lim[small].load()) {
+            std::lock_guard<std::mutex> lock(mu_lim);
+            if (sm > lim[small].load() &&
+                cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess)
+                lim[small].store(sm);
+        }
+        if (small) k_refresh_mu<T, 32, 4, 1><<<nblk, 128, sm, st>>>(im, ch, part_ll, write_state, err);
+        else k_refresh_mu<T, 64, 4, 4><<<nblk, 256, sm, st>>>(im, ch, part_ll, write_state, err);
+    }
     // the patch and its row transforms in shared memory (24 bytes per patch pixel)
     const size_t smem = 8 * (size_t)(((size_t)im.S * im.S + 1) / 2 * 2) + 16 * (size_t)im.S * im.S;
     static std::atomic<size_t> limit{48 * 1024};   // the dynamic shared-memory limit only grows

@@ -135,16 +135,6 @@ __device__ __forceinline__ void proposal(const Image& im, const Chain& ch, int m
     delta = r_new - r_old;
 }
 
-// phi_logterm with log phi! from the table of the first kLgamma counts: two
-// double lgamma per drawn pixel and sweep (about 200 FP64 operations each, at
-// 2 FP64 lanes per SM and cycle) took a quarter of the augmented 512 x 512
-// sweep.
-__device__ __forceinline__ double phi_logterm_tab(int phi, double lmu, double c, double is2, const double* lgam)
-{
-    const double d = c - (double)phi;
-    return -0.5 * d * d * is2 + (double)phi * lmu - (phi < kLgamma ? lgam[phi] : lgamma((double)phi + 1.0));
-}
-
 // Photon-count step of the augmented sampler for one patch (camera grid), one
 // thread's share: draws phi_n ~ p(phi | w_n, mu_n) (Philox counter (n, t,
 // chain, 1)) for the camera pixels centred on the patch; returns the warp's

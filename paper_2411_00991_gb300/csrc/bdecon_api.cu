@@ -174,6 +174,28 @@ struct Alloc {
 
 bool finite_pos(double x) { return std::isfinite(x) && x > 0.0; }
 
+// Index of the first value that is not finite (positive: nor > 0), -1 if all
+// are: bit patterns compared a block at a time, without a branch per value.
+template <typename T, typename U>
+int64_t first_bad(const T* v, int64_t n, bool positive)
+{
+    const U inf = sizeof(T) == 4 ? (U)0x7f800000u : (U)0x7ff0000000000000ull, sign = (U)1 << (8 * sizeof(T) - 1);
+    for (int64_t b = 0; b < n; b += 1024) {
+        const int64_t e = std::min<int64_t>(n, b + 1024);
+        U bad = 0;
+        for (int64_t k = b; k < e; ++k) {
+            U u;
+            std::memcpy(&u, v + k, sizeof u);
+            // positive and finite: 0 < u < inf as an unsigned pattern
+            bad |= positive ? (U)((U)(u - 1) >= (U)(inf - 1)) : (U)((u & ~sign) >= inf);
+        }
+        if (!bad) continue;
+        for (int64_t k = b; k < e; ++k)
+            if (!std::isfinite(v[k]) || (positive && !(v[k] > (T)0))) return k;
+    }
+    return -1;
+}
+
 bdecon_status validate(const bdecon_problem& p, int idx)
 {
     if (p.H < 1 || p.W < 1 || p.H > 16384 || p.W > 16384)
@@ -207,19 +229,19 @@ bdecon_status validate(const bdecon_problem& p, int idx)
     }
     if (!(s > 0.0)) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: PSF sums to zero", idx);
     const int64_t n = (int64_t)p.H * p.W;
-    for (int64_t k = 0; k < n; ++k)
-        if (!std::isfinite(p.image[k])) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: image[%lld] not finite", idx, (long long)k);
+    int64_t at = first_bad<float, uint32_t>(p.image, n, false);
+    if (at >= 0) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: image[%lld] not finite", idx, (long long)at);
     if (p.gain_map) {
-        for (int64_t k = 0; k < n; ++k)
-            if (!finite_pos(p.gain_map[k])) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: gain_map[%lld] must be > 0", idx, (long long)k);
+        at = first_bad<float, uint32_t>(p.gain_map, n, true);
+        if (at >= 0) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: gain_map[%lld] must be > 0", idx, (long long)at);
     } else if (!finite_pos(p.gain)) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: gain must be > 0", idx);
     if (p.var_map) {
-        for (int64_t k = 0; k < n; ++k)
-            if (!finite_pos(p.var_map[k])) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: var_map[%lld] must be > 0", idx, (long long)k);
+        at = first_bad<float, uint32_t>(p.var_map, n, true);
+        if (at >= 0) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: var_map[%lld] must be > 0", idx, (long long)at);
     } else if (!finite_pos(p.read_var)) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: read_var must be > 0", idx);
     if (p.offset_map) {
-        for (int64_t k = 0; k < n; ++k)
-            if (!std::isfinite(p.offset_map[k])) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: offset_map not finite", idx);
+        if (first_bad<float, uint32_t>(p.offset_map, n, false) >= 0)
+            return fail(nullptr, BDECON_ERR_INVALID, "problem %d: offset_map not finite", idx);
     } else if (!std::isfinite(p.offset)) return fail(nullptr, BDECON_ERR_INVALID, "problem %d: offset not finite", idx);
     return BDECON_OK;
 }
@@ -807,9 +829,9 @@ size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainH
         ph.o_samp = ph.p.n_samples > 0 ? A.take(ts * nobj * (size_t)ph.p.n_samples * ph.p.n_chains) : 0;
         const bool adapt = ph.p.adapt_target > 0.0 && ph.p.burn_in > 0;
         ph.o_adapt = adapt ? A.take(16 * (size_t)ph.p.burn_in) : 0;
-        ph.o_lgam = (ph.p.flags & BDECON_FLAG_AUGMENTED) ? A.take(8 * (size_t)kLgamma) : 0;
+        ph.o_lgam = A.take(8 * (size_t)kLgamma);
         const size_t nblk = (npix + kRedThreads - 1) / kRedThreads;
-        ph.scr_doubles = std::max(nblk + (size_t)ph.n_patches + 8, nblk + 8 + 2 * (size_t)kMaxS * kMaxS) + 8;
+        ph.scr_doubles = std::max(std::max(nblk, (size_t)refresh_blocks(ph.H, ph.W, ph.f)) + (size_t)ph.n_patches + 8, nblk + 8 + 2 * (size_t)kMaxS * kMaxS) + 8;
         ph.o_scr = A.take(8 * ph.scr_doubles);
         scr_max = std::max(scr_max, ph.scr_doubles);
         up = std::max(up, std::max(16 * npix + 8 * (size_t)ph.L * ph.L, 8 * nobj));
@@ -1055,8 +1077,8 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
         im.sample_every = ph.p.sample_every > 0 ? ph.p.sample_every : 1;
         im.n_samples = ph.p.n_samples;
         im.adapt_fac = ph.o_adapt ? (const double*)(A + ph.o_adapt) : nullptr;
-        im.lgam = ph.o_lgam ? (const double*)(A + ph.o_lgam) : nullptr;
-        if (im.lgam) launch_lgamma((double*)(A + ph.o_lgam), h->st, &h->launches);
+        im.lgam = (const double*)(A + ph.o_lgam);
+        launch_lgamma((double*)(A + ph.o_lgam), h->st, &h->launches);
     }
     h->chains.resize(h->chh.size());
     for (int k = 0; k < n; ++k) {
@@ -1758,8 +1780,8 @@ bdecon_status bdecon_set_state(bdecon_handle* h, int32_t p, int32_t c, const dou
     if (sweeps < 0 || sweeps > h->max_sweeps) return fail(h, BDECON_ERR_INVALID, "sweep counter %lld out of range", (long long)sweeps);
     const ProbHost& ph0 = h->probs[p];
     const int64_t n = (int64_t)ph0.Ho * ph0.Wo;
-    for (int64_t k = 0; k < n; ++k)
-        if (!(std::isfinite(rho[k]) && rho[k] > 0.0)) return fail(h, BDECON_ERR_INVALID, "rho[%lld] must be finite and > 0", (long long)k);
+    const int64_t at = first_bad<double, uint64_t>(rho, n, true);
+    if (at >= 0) return fail(h, BDECON_ERR_INVALID, "rho[%lld] must be finite and > 0", (long long)at);
     s = check_device(h);
     if (s != BDECON_OK) return s;
     CK(h, cudaMemcpyAsync(h->d_up, rho, 8 * (size_t)n, cudaMemcpyHostToDevice, h->st));
