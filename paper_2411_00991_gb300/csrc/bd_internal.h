@@ -257,21 +257,22 @@ constexpr uint32_t kRowChgMask = (1u << kRowChgBits) - 1u;
 constexpr int kRowMapBytes = 384;    // three TMA tensor maps per chain: mu, then cumulants or photon counts
 // columns of a run's window box: L + V - 1 cells from a start rounded down to
 // a multiple of 4 cells; a box side is at most 256 elements, 4 per cell
-__host__ __device__ inline int rows_box_w(int L, int V) { return (L + V + 5) & ~3; }
+// (L: side of the camera window; with f lattice cells a camera pixel the V classes span (V - 1 + f - 1) / f more columns)
+__host__ __device__ inline int rows_box_w(int L, int V, int f) { return (L + (V + f - 2) / f + 6) & ~3; }
 __host__ __device__ inline int rows_ring_slots(int V) { return V <= 4 ? 4 : V <= 8 ? 8 : 16; }
 struct RowsSmem {
     size_t K, tw, ent, ring, red, mu, cum, cum2, spec, total;
 };
-__host__ __device__ inline RowsSmem rows_smem(int L, int S, int V, int G, int nwt, int n_tw, int nhalf0, bool aug,
+__host__ __device__ inline RowsSmem rows_smem(int L, int Le, int f, int V, int G, int nwt, int n_tw, int nhalf0, bool aug,
                                               int spec_entries)
 {
     RowsSmem p;
     size_t o = 0;
-    const size_t cells = (size_t)rows_box_w(L, V) * L;
+    const size_t cells = (size_t)rows_box_w(L, V, f) * L;
     p.mu = o; o += al128(4 * cells);
     p.cum = o; o += al128((aug ? 4 : 16) * cells);
     p.cum2 = o; o += aug ? 0 : al128(8 * cells);
-    p.K = o; o += al16((size_t)L * L * 4);
+    p.K = o; o += al16((size_t)Le * Le * 4);
     p.tw = o; o += al16((size_t)n_tw * 8);
     p.ent = o; o += al16((size_t)nhalf0 * 8);
     p.ring = o; o += 64 * 16;
@@ -316,7 +317,7 @@ cudaError_t launch_sweep(const SweepArgs& a, int grid, int threads, size_t smem,
 template <typename T>
 int sweep_blocks_per_sm(int threads, size_t smem, bool aug, bool fine, int stg, bool solo, bool lean);
 cudaError_t launch_sweep_rows(const SweepArgs& a, int grid, int threads, size_t smem, cudaStream_t st);
-int rows_blocks_per_sm(bool aug, int vg, int threads, size_t smem);
+int rows_blocks_per_sm(bool aug, bool fine, int vg, int threads, size_t smem);
 // zero every chain's progress words and trace partials
 void launch_reset(const Image* d_imgs, const Chain* d_chains, int n_chains, int n_slots, cudaStream_t st,
                   int64_t* launches);

@@ -84,7 +84,10 @@ struct RowEnt { int kl; float wa; };
 
 constexpr uint32_t kUndecided = 0x80000000u;   // in place of a run's accept mask: the right tile is not done
 
-template <bool AUG, int VG, int MAXT, int MINB>
+// FINE: an object lattice f times finer than the camera.  A class offset v is
+// then a lattice column; its window starts at camera column (j0 + v) / f, and
+// its kernel entries depend on the phase (j0 + v) mod f.
+template <bool AUG, bool FINE, int VG, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
 {
     using P = Prec<float>;
@@ -124,17 +127,19 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
     const int t0 = *ch.tdev;
     const int tl = (int)blockIdx.x - ch.cta_base;
     const int ti = tl / ch.ntj, tj = tl - (tl / ch.ntj) * ch.ntj;
-    const int S = im.S, L = im.L, R2 = 2 * im.R, LL = L * L;
+    // L: side of an update's camera window; f, Le: lattice cells a camera pixel, side of the kernel
+    const int S = im.S, L = FINE ? im.Lc : im.L, LL = L * L, f = FINE ? im.f : 1;
+    auto Le = [&]() { return FINE ? im.Le : L; };
     const int pi0 = ti * ch.tpi, pj0 = tj * ch.tpj;
     const int tw_ = min(ch.tpj, im.npj - pj0), th_ = min(ch.tpi, im.npi - pi0), npt = th_ * tw_;
     // the block: G update teams of NT threads, each scoring VG classes of a run
     const int NT = im.team, G = blockDim.x / NT, V = G * VG, nwt = NT >> 5;
     const int g = tid / NT, lt = tid - g * NT, gw = lt >> 5, vb = g * VG;
     const int RN = (S + V - 1) / V;                 // runs per class row
-    const int BW = rows_box_w(L, V);
+    const int BW = rows_box_w(L, V, f);
     const int VR = rows_ring_slots(V), DP = 32 / VR; // proposal ring: slots per patch-run, patch-runs per draw
     const Shape& sh0 = im.shape[0];
-    const RowsSmem sp = rows_smem(L, S, V, G, nwt, im.n_tw, sh0.nhalf, AUG, a.resident ? im.max_nhalf : 0);
+    const RowsSmem sp = rows_smem(L, Le(), f, V, G, nwt, im.n_tw, sh0.nhalf, AUG, a.resident ? im.max_nhalf : 0);
     float* Ks = reinterpret_cast<float*>(smem + sp.K);
     float2* tws = reinterpret_cast<float2*>(smem + sp.tw);
     RowEnt* ent0 = reinterpret_cast<RowEnt*>(smem + sp.ent);
@@ -153,7 +158,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
     const Dat4<float>* dat_g = dat<float>(im);
 
     for (int k = tid; k <= RN; k += blockDim.x) s_v0[k] = (short)(k * S / RN);   // first class of each run
-    for (int k = tid; k < LL; k += blockDim.x) Ks[k] = im.Ke32[k];
+    for (int k = tid; k < Le() * Le(); k += blockDim.x) Ks[k] = im.Ke32[k];
     for (int k = tid; k < im.n_tw; k += blockDim.x) tws[k] = reinterpret_cast<const float2*>(im.tw32)[k];
     for (int k = tid; k < sh0.nhalf; k += blockDim.x)   // full patches' entries (others are read from global memory)
         ent0[k] = {im.ent_kl[sh0.ent_off + k] | (im.ent_m32[sh0.ent_off + k] > 1.0f ? (int)0x80000000 : 0),
@@ -324,9 +329,11 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                         float* rdL = rdS + V * nwt;
                         float* rdA = rdL + V * nwt;
                         uint32_t* rdB = reinterpret_cast<uint32_t*>(rdA + G * nwt);
-                        const int dx = (j0 - R2) & 3;
+                        const int xb = j0 / f - (L - 1), y0 = i / f - (L - 1), dx = xb & 3;   // window of the run's first class
+                        // (FINE) kernel rows and columns of a window cell: f kr + po, f kc + po - phase
+                        const int po = FINE ? Le() - 1 - f * (L - 1) : 0;
                         auto copy_window = [&]() {   // one thread
-                            const int x0 = (j0 - R2) & ~3, y0 = i - R2;
+                            const int x0 = xb & ~3;
                             if (fence_copy) fence_proxy_async_all();
                             mbar_arrive_expect_tx(&s_bar, (uint32_t)(AUG ? 8 : 28) * (uint32_t)(BW * L));
                             tma_load_2d(wmu, tmap, x0, y0, &s_bar);
@@ -452,21 +459,36 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
 #pragma unroll
                                 for (int k = 0; k < NL; ++k) acc[k] = 0.0f;
                                 uint32_t badL = 0;
-                                int kc = kc0, idx = idx0 + dx + vb;
+                                int kc = kc0, idx = idx0 + dx + (FINE ? 0 : vb);
+                                int cs[FINE ? VG : 1], qo[FINE ? VG : 1], kr = FINE ? lt / L : 0;
+                                if constexpr (FINE) {
+#pragma unroll
+                                    for (int k = 0; k < VG; ++k) {
+                                        cs[k] = (j0 + vb + k) / f - j0 / f;
+                                        qo[k] = po - (j0 + vb + k) % f;
+                                    }
+                                }
+                                // box index and kernel entry (0 outside the kernel) of this cell for class k
+                                auto cell = [&](int k) { return idx + (FINE ? cs[FINE ? k : 0] : k); };
+                                auto kern = [&](int c, int k) -> float {
+                                    if constexpr (!FINE) return Ks[c];
+                                    const int p = f * kr + po - i % f, q = f * kc + qo[FINE ? k : 0];
+                                    return (unsigned)p < (unsigned)im.Le && (unsigned)q < (unsigned)im.Le ? Ks[p * im.Le + q] : 0.0f;
+                                };
                                 for (int c = lt; c < LL; c += NT) {
-                                    const float K = Ks[c];
+                                    const float K0 = FINE ? 0.0f : Ks[c];
                                     float val[VG];
                                     bool slow = false;
 #pragma unroll
                                     for (int k = 0; k < VG; ++k) {
-                                        const float xk = mul_rn(del[k], K);
+                                        const float xk = mul_rn(del[k], FINE ? kern(c, k) : K0);
                                         if constexpr (AUG) {
-                                            const float d = xk / wmu[idx + k];
-                                            val[k] = wphi[idx + k] * log1p_small(d) - xk;
+                                            const float d = xk / wmu[cell(k)];
+                                            val[k] = wphi[cell(k)] * log1p_small(d) - xk;
                                             slow = slow || !(fabsf(d) <= 0.05f);
                                         } else {
-                                            const float d = xk * P::rcp(wmu[idx + k]);
-                                            val[k] = cgf_delta(xk, log1p_small(d), wcum[idx + k], wcum2[idx + k]);
+                                            const float d = xk * P::rcp(wmu[cell(k)]);
+                                            val[k] = cgf_delta(xk, log1p_small(d), wcum[cell(k)], wcum2[cell(k)]);
                                             slow = slow || !(fabsf(d) <= 0.05f);
                                         }
                                     }
@@ -476,17 +498,22 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                                         uint32_t todo = 0;
 #pragma unroll
                                         for (int k = 0; k < VG; ++k) {
-                                            const float mu = wmu[idx + k];
+                                            const float mu = wmu[cell(k)];
                                             if (!(mu > 0.0f)) val[k] = 0.0f;
                                             else todo |= 1u << k;
                                         }
                                         while (todo) {
                                             const int k = __ffs(todo) - 1;
                                             todo &= todo - 1;
-                                            float dk = del[0];
+                                            float dk = del[0], Kk = FINE ? kern(c, 0) : K0;
+                                            int ix = cell(0);
 #pragma unroll
-                                            for (int z = 1; z < VG; ++z) dk = k == z ? del[z] : dk;
-                                            const float mu = wmu[idx + k], xk = mul_rn(dk, K);
+                                            for (int z = 1; z < VG; ++z) {
+                                                dk = k == z ? del[z] : dk;
+                                                ix = k == z ? cell(z) : ix;
+                                                if constexpr (FINE) Kk = k == z ? kern(c, z) : Kk;
+                                            }
+                                            const float mu = wmu[ix], xk = mul_rn(dk, Kk);
                                             float y;
                                             if constexpr (AUG) {
                                                 const float d = xk / mu;
@@ -494,16 +521,16 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                                                     badL |= 1u << k;
                                                     y = 0.0f;
                                                 } else {
-                                                    y = wphi[idx + k] * log1p_cum(d) - xk;
+                                                    y = wphi[ix] * log1p_cum(d) - xk;
                                                 }
                                             } else {
                                                 const float d = xk * P::rcp(mu);
                                                 if (fabsf(d) <= kCumEval) {
-                                                    y = cgf_delta(xk, log1p_cum(d), wcum[idx + k], wcum2[idx + k]);
+                                                    y = cgf_delta(xk, log1p_cum(d), wcum[ix], wcum2[ix]);
                                                 } else {
-                                                    const int kr = c / L;
+                                                    const int rr = c / L;
                                                     const Dat4<float> dv =
-                                                        dat_g[(size_t)(i - R2 + kr) * im.W + (j0 + vb + k - R2 + (c - kr * L))];
+                                                        dat_g[(size_t)(y0 + rr) * im.W + ((j0 + vb + k) / f - (L - 1) + (c - rr * L))];
                                                     int b = 0;
                                                     y = dl_pixel_call(mu, xk, dv.c, dv.is2, dv.beta, &b);
                                                     badL |= b ? 1u << k : 0u;
@@ -517,9 +544,11 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                                     for (int k = 0; k < VG; ++k) acc[k] += val[k];
                                     kc += dkc;
                                     idx += didx;
+                                    if constexpr (FINE) kr += NT / L;
                                     if (kc >= L) {
                                         kc -= L;
                                         idx += dwrap;
+                                        if constexpr (FINE) ++kr;
                                     }
                                 }
                                 const float s = warp_sum_many<NL>(acc);
@@ -651,11 +680,18 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                             ++n_acc;
                             const float delta = ring[rbase + fin].w;
                             for (int c = tid; c < LL; c += blockDim.x) {
-                                const int kr = c / L, kc = c - kr * L, idx = kr * BW + kc + dx + fin;
+                                const int kr = c / L, kc = c - kr * L, xf = (j0 + fin) / f - (L - 1);
+                                const int idx = kr * BW + kc + dx + (xf - xb);
                                 const float old = wmu[idx];
                                 if (!(old > 0.0f)) continue;   // outside the frame
-                                const size_t gx = (size_t)(i - R2 + kr) * im.mu_pitch + (j0 + fin - R2 + kc);
-                                const float xk = mul_rn(delta, Ks[c]), nmu = add_rn(old, xk);
+                                int kw = c;
+                                if constexpr (FINE) {
+                                    const int p = f * kr + po - i % f, q = f * kc + po - (j0 + fin) % f;
+                                    if ((unsigned)p >= (unsigned)im.Le || (unsigned)q >= (unsigned)im.Le) continue;   // outside the kernel
+                                    kw = p * im.Le + q;
+                                }
+                                const size_t gx = (size_t)(y0 + kr) * im.mu_pitch + (xf + kc);
+                                const float xk = mul_rn(delta, Ks[kw]), nmu = add_rn(old, xk);
                                 __stcg(mu_g + gx, nmu);
                                 wmu[idx] = nmu;
                                 if constexpr (!AUG) {
@@ -664,7 +700,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                                     if (fabsf(d) <= kCumShift) {
                                         nq = cgf_shift(wcum[idx], wcum2[idx], log1p_small(d));
                                     } else {
-                                        const Dat4<float> dv = dat_g[(size_t)(i - R2 + kr) * im.W + (j0 + fin - R2 + kc)];
+                                        const Dat4<float> dv = dat_g[(size_t)(y0 + kr) * im.W + (xf + kc)];
                                         nq = photon_cumulants_call(nmu, dv.c, dv.is2, dv.beta);
                                     }
                                     __stcg(ch.cum + gx, nq.a);
@@ -733,20 +769,23 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
 
 namespace {
 
-template <bool AUG>
+template <bool AUG, bool FINE>
 const void* rows_fn_of(int vg, int threads)
 {
     switch (vg) {
-    case 1: return (const void*)k_sweep_rows<AUG, 1, 320, 2>;
-    case 4: return (const void*)k_sweep_rows<AUG, 4, 128, 5>;
-    case 5: return (const void*)k_sweep_rows<AUG, 5, 128, 5>;
-    default: return threads <= 224 ? (const void*)k_sweep_rows<AUG, 3, 224, 4> : (const void*)k_sweep_rows<AUG, 3, 256, 3>;
+    case 1: return (const void*)k_sweep_rows<AUG, FINE, 1, 320, 2>;
+    case 4: return (const void*)k_sweep_rows<AUG, FINE, 4, 128, 5>;
+    case 5: return (const void*)k_sweep_rows<AUG, FINE, 5, 128, 5>;
+    default:
+        return threads <= 224 ? (const void*)k_sweep_rows<AUG, FINE, 3, 224, 4> : (const void*)k_sweep_rows<AUG, FINE, 3, 256, 3>;
     }
 }
 
-const void* rows_fn(bool aug, int vg, int threads)
+// (the augmented sampler on a finer lattice keeps the general form)
+const void* rows_fn(bool aug, bool fine, int vg, int threads)
 {
-    return aug ? rows_fn_of<true>(vg, threads) : rows_fn_of<false>(vg, threads);
+    return aug ? rows_fn_of<true, false>(vg, threads)
+               : fine ? rows_fn_of<false, true>(vg, threads) : rows_fn_of<false, false>(vg, threads);
 }
 
 cudaError_t rows_smem_limit(const void* fn, size_t smem)
@@ -767,7 +806,7 @@ cudaError_t launch_sweep_rows(const SweepArgs& a, int grid, int threads, size_t 
 {
     SweepArgs args = a;
     void* kargs[] = {&args};
-    const void* fn = rows_fn(a.aug != 0, a.row_vg, threads);
+    const void* fn = rows_fn(a.aug != 0, a.fine != 0, a.row_vg, threads);
     cudaError_t e = rows_smem_limit(fn, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -783,9 +822,9 @@ cudaError_t launch_sweep_rows(const SweepArgs& a, int grid, int threads, size_t 
     return cudaLaunchKernelExC(&cfg, fn, kargs);
 }
 
-int rows_blocks_per_sm(bool aug, int vg, int threads, size_t smem)
+int rows_blocks_per_sm(bool aug, bool fine, int vg, int threads, size_t smem)
 {
-    const void* fn = rows_fn(aug, vg, threads);
+    const void* fn = rows_fn(aug, fine, vg, threads);
     int n = 0;
     if (rows_smem_limit(fn, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem) != cudaSuccess) {

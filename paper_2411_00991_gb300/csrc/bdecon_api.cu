@@ -331,17 +331,17 @@ int occupancy(int prec, int threads, size_t smem, bool aug, bool fine, int stg, 
     return n;
 }
 
-int occupancy_rows(bool aug, int vg, int threads, size_t smem)
+int occupancy_rows(bool aug, bool fine, int vg, int threads, size_t smem)
 {
     static std::mutex mu;
     static std::map<std::vector<long long>, int> memo;
     int dev = 0;
     cudaGetDevice(&dev);
-    const std::vector<long long> key = {dev, aug ? 1 : 0, vg, threads, (long long)smem};
+    const std::vector<long long> key = {dev, aug ? 1 : 0, fine ? 1 : 0, vg, threads, (long long)smem};
     std::lock_guard<std::mutex> lock(mu);
     auto it = memo.find(key);
     if (it != memo.end()) return it->second;
-    const int n = rows_blocks_per_sm(aug, vg, threads, smem);
+    const int n = rows_blocks_per_sm(aug, fine, vg, threads, smem);
     if (n > 0) memo[key] = n;
     return n;
 }
@@ -430,7 +430,7 @@ bool encode_window_map(const ProbHost& ph, void* base, int per, int bw, CUtensor
     const cuuint32_t es[2] = {1, 1};
     const cuuint64_t dims[2] = {(cuuint64_t)per * ph.W, (cuuint64_t)ph.H};
     const cuuint64_t strides[1] = {(cuuint64_t)per * 4 * ph.pitch};
-    const cuuint32_t box[2] = {(cuuint32_t)(per * bw), (cuuint32_t)ph.L};
+    const cuuint32_t box[2] = {(cuuint32_t)(per * bw), (cuuint32_t)ph.Lc};
     return enc(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -451,8 +451,8 @@ void place_items(std::vector<PlanItem*>& items, Group& g)
     g.grid = base;
 }
 
-// Plan of the row-run form, where it applies: float problems on the camera
-// grid of one PSF side, stride and team, S >= 3 (a class row of one or two
+// Plan of the row-run form, where it applies: float problems of one PSF side,
+// lattice, stride and team (augmented ones on the camera grid only), S >= 3 (a class row of one or two
 // classes has nothing to score together), the run's window box within the TMA
 // limit, and no other form asked for (block warps, streaming, staging, lean).
 //
@@ -474,12 +474,12 @@ void place_items(std::vector<PlanItem*>& items, Group& g)
 bool plan_rows(int precision, int sms, std::vector<PlanItem*>& items, Group& g)
 {
     g.rows = false;
-    if (precision != BDECON_FP32 || g.fine || g.user_warps || g.streamed || !g.no_stage || g.lean_mode != -1) return false;
+    if (precision != BDECON_FP32 || (g.fine && g.aug) || g.user_warps || g.streamed || !g.no_stage || g.lean_mode != -1) return false;
     const PlanItem& i0 = *items[0];
-    const int L = i0.ph->L, S = i0.ph->S, team = i0.team;
+    const int L = i0.ph->Lc, Le = i0.ph->Le, f = i0.ph->f, S = i0.ph->S, team = i0.team;
     long long patches = 0;
     for (const PlanItem* it : items) {
-        if (it->ph->L != L || it->ph->S != S || it->team != team) return false;
+        if (it->ph->Lc != L || it->ph->Le != Le || it->ph->f != f || it->ph->S != S || it->team != team) return false;
         patches += (long long)it->chains.size() * it->ph->n_patches;
     }
     if (S < 3) return false;
@@ -496,7 +496,7 @@ bool plan_rows(int precision, int sms, std::vector<PlanItem*>& items, Group& g)
     for (const auto& shape : shapes) {
         const int VG = shape.first, G = shape.second;
         const int V = G * VG, threads = G * team, RN = (S + V - 1) / V;
-        if (4 * rows_box_w(L, V) > 256) continue;
+        if (4 * rows_box_w(L, V, f) > 256) continue;
         for (PlanItem* it : items)
             if (!it->user) it->tpi = it->tpj = 1;
         for (;;) {
@@ -505,13 +505,13 @@ bool plan_rows(int precision, int sms, std::vector<PlanItem*>& items, Group& g)
             size_t smem = 0;
             int tot = 0, area = 1;
             for (const PlanItem* it : items) {
-                smem = std::max(smem, rows_smem(L, S, V, G, team / 32, it->ph->n_tw, it->ph->shape[0].nhalf, g.aug,
+                smem = std::max(smem, rows_smem(L, Le, f, V, G, team / 32, it->ph->n_tw, it->ph->shape[0].nhalf, g.aug,
                                                 one ? it->ph->max_nhalf : 0).total);
                 tot += item_blocks(*it);
                 area = std::max(area, std::min(it->tpi, it->ph->npi) * std::min(it->tpj, it->ph->npj));
             }
             if (smem > kMaxSmem) break;
-            const int bps = occupancy_rows(g.aug, VG, threads, smem);
+            const int bps = occupancy_rows(g.aug, g.fine, VG, threads, smem);
             if (bps > 0 && tot <= bps * sms) {
                 const int per_sm = (tot + sms - 1) / sms;
                 const double w = (double)per_sm * threads / 32;
@@ -535,7 +535,7 @@ bool plan_rows(int precision, int sms, std::vector<PlanItem*>& items, Group& g)
     }
     const int VG = best_shape.first, V = best_shape.second * VG, threads = best_shape.second * team;
     g.rmaps.clear();
-    const int bw = rows_box_w(L, V);
+    const int bw = rows_box_w(L, V, f);
     for (const PlanItem* it : items)
         for (const Chain* ch : it->chains) {
             CUtensorMap m[3];

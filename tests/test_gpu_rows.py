@@ -52,10 +52,13 @@ CASES = [
     dict(H=70, W=65, L=31, sigma=4.0, peak=5.0),            # eight-warp teams
     dict(H=60, W=47, L=55, sigma=8.0),                      # the widest window box
     dict(H=64, W=66, L=59, sigma=9.0),                      # above it: the general form
+    dict(H=20, W=22, L=7, subpixel=2),                      # finer lattices: every phase of the kernel
+    dict(H=15, W=17, L=5, subpixel=3, stride=9, maps=True),
+    dict(H=40, W=33, L=25, sigma=5.0, subpixel=2, n_chains=2),
 ]
 
 
-@pytest.mark.parametrize("kw", CASES, ids=lambda kw: "%dx%dL%d" % (kw["H"], kw["W"], kw["L"]))
+@pytest.mark.parametrize("kw", CASES, ids=lambda kw: "%dx%dL%df%d" % (kw["H"], kw["W"], kw["L"], kw.get("subpixel", 1)))
 @pytest.mark.parametrize("augmented", [False, True])
 def test_rows_are_bit_identical_to_the_general_form(kw, augmented):
     p = synth.small_problem(seed=17, refresh_every=4, burn_in=2, **kw)
