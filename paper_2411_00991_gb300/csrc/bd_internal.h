@@ -260,6 +260,9 @@ constexpr int kRowMapBytes = 384;    // three TMA tensor maps per chain: mu, the
 // (L: side of the camera window; with f lattice cells a camera pixel the V classes span (V - 1 + f - 1) / f more columns)
 __host__ __device__ inline int rows_box_w(int L, int V, int f) { return (L + (V + f - 2) / f + 6) & ~3; }
 __host__ __device__ inline int rows_ring_slots(int V) { return V <= 4 ? 4 : V <= 8 ? 8 : 16; }
+// slots drawn at a time (half of the ring): fewer for VG = 4, whose widest
+// windows then leave room for a fifth block per SM (L = 31)
+__host__ __device__ constexpr int rows_ring_half(int VG) { return VG == 4 ? 16 : 32; }
 struct RowsSmem {
     size_t K, tw, ent, ring, red, mu, cum, cum2, spec, total;
 };
@@ -275,7 +278,7 @@ __host__ __device__ inline RowsSmem rows_smem(int L, int Le, int f, int V, int G
     p.K = o; o += al16((size_t)Le * Le * 4);
     p.tw = o; o += al16((size_t)n_tw * 8);
     p.ent = o; o += al16((size_t)nhalf0 * 8);
-    p.ring = o; o += 64 * 16;
+    p.ring = o; o += (size_t)2 * rows_ring_half(V / G) * 16;
     p.red = o; o += al16((size_t)2 * nwt * 3 * (V + G) * 4);
     p.spec = o; o += al16((size_t)spec_entries * 8);
     p.total = o;

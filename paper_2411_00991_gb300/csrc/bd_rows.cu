@@ -136,8 +136,9 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
     const int NT = im.team, G = blockDim.x / NT, V = G * VG, nwt = NT >> 5;
     const int g = tid / NT, lt = tid - g * NT, gw = lt >> 5, vb = g * VG;
     const int RN = (S + V - 1) / V;                 // runs per class row
+    constexpr int RH = rows_ring_half(VG);          // ring slots drawn at a time
     const int BW = rows_box_w(L, V, f);
-    const int VR = rows_ring_slots(V), DP = 32 / VR; // proposal ring: slots per patch-run, patch-runs per draw
+    const int VR = rows_ring_slots(V), DP = RH / VR; // proposal ring: slots per patch-run, patch-runs per draw
     const Shape& sh0 = im.shape[0];
     const RowsSmem sp = rows_smem(L, Le(), f, V, G, nwt, im.n_tw, sh0.nhalf, AUG, a.resident ? im.max_nhalf : 0);
     float* Ks = reinterpret_cast<float*>(smem + sp.K);
@@ -671,7 +672,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                                 }
                             }
                             const uint32_t mask = s_mask;
-                            if (lo == 0 && ahead && epos == 0 && warp == 0) draw(e + DP, DP, ebase ^ 32);
+                            if (lo == 0 && ahead && epos == 0 && warp == 0) draw(e + DP, DP, ebase ^ RH);
                             if (!mask) break;
                             // write the accepted update: window (global and staged), spectrum
                             const int fin = __ffs(mask) - 1;
@@ -728,10 +729,10 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                         if (ahead) {
                             if (++epos == DP) {
                                 epos = 0;
-                                ebase ^= 32;
+                                ebase ^= RH;
                             }
                         } else {
-                            ebase ^= 32;
+                            ebase ^= RH;
                         }
                     }
                 }
