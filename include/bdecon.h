@@ -353,7 +353,10 @@ bdecon_status bdecon_get_staging(bdecon_handle* h, int32_t p, int32_t* staged);
  * for PSF windows of more than 256 pixels (side 17 and up; measured faster
  * there, slower for smaller windows); 0: never; 1: wherever eligible.
  * bdecon_autotune tries both.  Results do not change.
- * bdecon_get_lean reports whether problem p's launch group runs it.        */
+ * With -1 float problems run, where it applies, the row-run form, which
+ * scores runs of classes at once; 0 and 1 keep them in the class-by-class
+ * forms.  bdecon_get_lean reports whether problem p's launch group runs the
+ * lean form.                                                               */
 bdecon_status bdecon_set_lean(bdecon_handle* h, int32_t mode);
 bdecon_status bdecon_get_lean(bdecon_handle* h, int32_t p, int32_t* lean);
 

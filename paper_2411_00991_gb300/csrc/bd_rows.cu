@@ -36,8 +36,9 @@
 // and window bounds worked out once per run; DRAM reads per update 31 -> 8 KB
 // on the 2048 x 2048 frame (L = 31).  ms per sweep, before and after (50, 2 and
 // 10 sweeps of long chains, with refresh and read-out): 512 x 512 L = 17 1.29
-// and 0.91; 2048 x 2048 L = 31 x 4 chains 189 and 102; six frames 128..768
-// x 4 chains 52 and 24; 64 x 64 L = 9 0.30 and 0.12.
+// and 0.91; 2048 x 2048 L = 31 x 4 chains 189 and 97; six frames 128..768
+// x 4 chains 52 and 22; 64 x 64 L = 9 0.30 and 0.12; 150 x 150 on a twice finer
+// lattice 1.13 and 0.40.
 #include <map>
 #include <mutex>
 

@@ -671,7 +671,26 @@ bool plan_general(int precision, int sms, std::vector<PlanItem*>& items, Group& 
 // 512 x 512 L = 17 50 -> 34).
 bool plan_items(int precision, int sms, std::vector<PlanItem*>& items, Group& g, std::string& err)
 {
-    if (plan_rows(precision, sms, items, g)) return true;
+    if (plan_rows(precision, sms, items, g)) {
+        // Augmented, one patch a block and a team of one or two warps: the
+        // general form's one-team plan, where all its blocks fit, keeps ahead (its
+        // whole sweep is as short as the count step that all neighbours share):
+        // 512 x 512 L = 13 0.95 against 1.03 ms a sweep, 400 x 400 L = 11 0.58
+        // against 0.63, 300 x 300 L = 9 x 2 chains 0.65 against 0.75; with three
+        // warps or more teams a block, or tiles of several patches, the row runs
+        // are ahead (512 x 512 L = 17 1.38 against 1.27, 256 x 256 L = 9 0.39
+        // against 0.28).
+        bool one = g.aug && g.threads <= 64;
+        for (const PlanItem* it : items) one = one && it->tpi == 1 && it->tpj == 1 && g.threads == it->team;
+        if (!one) return true;
+        Group q = g;
+        std::string err2;
+        if (plan_general(precision, sms, items, q, err2) && q.solo) {
+            g = q;
+            return true;
+        }
+        return plan_rows(precision, sms, items, g);
+    }
     if (precision == BDECON_FP64 && !g.streamed && g.no_stage) {
         auto cost = [&](const Group& q) {
             int area = 1;
