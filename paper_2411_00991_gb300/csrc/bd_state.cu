@@ -266,7 +266,7 @@ template void launch_init_rho<double>(const Image&, const Chain&, const double*,
 // sums RJ pixels TY rows apart, so a kernel entry is loaded once for RJ
 // products.  Bound by the FP64 unit (half a lane a cycle per sub-partition):
 // L^2 products and about 170..290 operations of the photon sum a pixel; 1024 x
-// 1024, L = 25, with the cumulants: 4.2 -> 2.1 ms.  Small frames take 128-pixel
+// 1024, L = 25: with the cumulants 4.2 -> 1.9 ms, without 3.1 -> 1.6.  Small frames take 128-pixel
 // tiles, one pixel a thread, to reach more SMs.
 __device__ __forceinline__ double block_sum_n(double v, double* sh, int n)
 {
