@@ -360,6 +360,14 @@ bdecon_status bdecon_get_staging(bdecon_handle* h, int32_t p, int32_t* staged);
 bdecon_status bdecon_set_lean(bdecon_handle* h, int32_t mode);
 bdecon_status bdecon_get_lean(bdecon_handle* h, int32_t p, int32_t* lean);
 
+/* Kernel form that problem p's launch group runs (outputs optional): *run
+ * classes scored at once by a block and *per_team of them by each of its
+ * update teams (row-run form; both 0 in the class-by-class forms), *resident
+ * 1 when tile state is held in shared memory (0: streamed from global),
+ * *one_team 1 for the one-patch one-team form.                             */
+bdecon_status bdecon_get_form(bdecon_handle* h, int32_t p, int32_t* run, int32_t* per_team,
+                              int32_t* resident, int32_t* one_team);
+
 /* Kernel launches issued by this handle since creation.                    */
 bdecon_status bdecon_launch_count(const bdecon_handle* h, int64_t* launches);
 

@@ -61,7 +61,7 @@ EXPORTS = ["bdecon_workspace_size", "bdecon_create", "bdecon_batch_create", "bde
            "bdecon_server_stop", "bdecon_set_grouping", "bdecon_autotune", "bdecon_set_graph",
            "bdecon_posterior_std", "bdecon_posterior_cv", "bdecon_get_samples", "bdecon_posterior_quantiles",
            "bdecon_get_steps", "bdecon_get_phi", "bdecon_set_staging", "bdecon_get_staging",
-           "bdecon_set_tuning_cache", "bdecon_set_lean", "bdecon_get_lean"]
+           "bdecon_set_tuning_cache", "bdecon_set_lean", "bdecon_get_lean", "bdecon_get_form"]
 
 JOB_QUEUED, JOB_RUNNING, JOB_DONE, JOB_FAILED = 0, 1, 2, 3
 
@@ -112,6 +112,7 @@ def load(build_if_missing: bool = True):
         "bdecon_get_staging": [H, i32, C.POINTER(i32)],
         "bdecon_set_lean": [H, i32],
         "bdecon_get_lean": [H, i32, C.POINTER(i32)],
+        "bdecon_get_form": [H, i32, C.POINTER(i32), C.POINTER(i32), C.POINTER(i32), C.POINTER(i32)],
         "bdecon_launch_count": [H, C.POINTER(i64)],
         "bdecon_set_timing": [H, i32],
         "bdecon_sweep_kernel_time": [H, dp, C.POINTER(i64)],
@@ -427,6 +428,12 @@ class Sampler:
         v = C.c_int32()
         self._ck(self.L.bdecon_get_lean(self.h, p, C.byref(v)))
         return int(v.value)
+
+    def form(self, p: int = 0):
+        """Kernel form of problem p's launch group: classes a run and per team (0: class by class), resident, one_team."""
+        run, per, res, one = C.c_int32(), C.c_int32(), C.c_int32(), C.c_int32()
+        self._ck(self.L.bdecon_get_form(self.h, p, C.byref(run), C.byref(per), C.byref(res), C.byref(one)))
+        return dict(run=run.value, per_team=per.value, resident=res.value, one_team=one.value)
 
     def staged(self, p: int = 0) -> int:
         """1 when problem p's launch group runs with window staging, else 0."""

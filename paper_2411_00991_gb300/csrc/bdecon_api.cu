@@ -1976,6 +1976,19 @@ bdecon_status bdecon_get_lean(bdecon_handle* h, int32_t p, int32_t* lean)
     return BDECON_OK;
 }
 
+bdecon_status bdecon_get_form(bdecon_handle* h, int32_t p, int32_t* run, int32_t* per_team, int32_t* resident,
+                              int32_t* one_team)
+{
+    if (!h) return fail(nullptr, BDECON_ERR_INVALID, "handle is NULL");
+    if (p < 0 || p >= (int)h->probs.size()) return fail(h, BDECON_ERR_INVALID, "problem index %d", p);
+    const Group& g = h->groups[h->prob_group[p]];
+    if (run) *run = g.rows ? g.rows_V : 0;
+    if (per_team) *per_team = g.rows ? g.rows_VG : 0;
+    if (resident) *resident = g.resident;
+    if (one_team) *one_team = g.solo ? 1 : 0;
+    return BDECON_OK;
+}
+
 namespace {
 
 // One autotuner trial: a segment of len sweeps in the current plan, timed
