@@ -252,6 +252,8 @@ __host__ __device__ inline SmemPlan smem_plan(int L, int f, int S, int n_tw, int
 // steps finished (19 bits: at most 64 sweeps x (64^2 + 1) steps a launch) above
 // a count of the runs that changed data, modulo 2^13.
 constexpr int kRowMaxV = 16;         // classes per run (ring slots of one patch-run)
+constexpr int kRowMaxTeams = 10;     // update teams per block (a bound of plan_rows; sizes per-team shared arrays)
+static_assert(kRowMaxTeams <= kRowMaxV && kRowMaxV / 3 <= kRowMaxTeams, "teams of a row-run block");
 constexpr int kRowChgBits = 13;
 constexpr uint32_t kRowChgMask = (1u << kRowChgBits) - 1u;
 constexpr int kRowMapBytes = 384;    // three TMA tensor maps per chain: mu, then cumulants or photon counts

@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
     __shared__ __align__(8) uint64_t s_bar;
     __shared__ __align__(16) uint32_t s_chd[sizeof(Chain) / 4];
     __shared__ __align__(16) uint32_t s_imd[sizeof(Image) / 4];
-    __shared__ double s_phid[AUG ? 8 : 1][8];
+    __shared__ double s_phid[AUG ? kRowMaxTeams : 1][8];   // [team][warp]
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     if (tid == 0) {

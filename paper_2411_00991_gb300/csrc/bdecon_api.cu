@@ -485,7 +485,7 @@ bool plan_rows(int precision, int sms, std::vector<PlanItem*>& items, Group& g)
     if (S < 3) return false;
     std::vector<std::pair<int, int>> shapes;   // (VG, G)
     if (team == 32 && patches <= 2LL * sms) {
-        shapes.push_back({1, std::min(S, 10)});
+        shapes.push_back({1, std::min(S, kRowMaxTeams)});
     } else {
         for (int G = 1; G <= std::min(std::max(1, 224 / team), std::min((S + 2) / 3, kRowMaxV / 3)); ++G) shapes.push_back({3, G});
         if (team == 128) shapes.insert(shapes.end(), {{4, 1}, {5, 1}});
