@@ -305,6 +305,9 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                 }
                 __syncthreads();
             }
+            // the next window copies read these counts through the async proxy,
+            // also where no neighbour's change would ask for the fence
+            fence_copy = true;
             publish(sweep_s, true);
         }
         uint32_t row_s = sweep_s;
