@@ -533,12 +533,17 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
                                                 if (fabsf(d) <= kCumEval) {
                                                     y = cgf_delta(xk, log1p_cum(d), wcum[ix], wcum2[ix]);
                                                 } else {
-                                                    const int rr = c / L;
-                                                    const Dat4<float> dv =
-                                                        dat_g[(size_t)(y0 + rr) * im.W + ((j0 + vb + k) / f - (L - 1) + (c - rr * L))];
-                                                    int b = 0;
-                                                    y = dl_pixel_call(mu, xk, dv.c, dv.is2, dv.beta, &b);
-                                                    badL |= b ? 1u << k : 0u;
+                                                    // (after a wait that failed the window is another run's, and a
+                                                    // positive mu no sign that the cell lies in the frame)
+                                                    const int rr = c / L, aa = y0 + rr;
+                                                    const int bb = (j0 + vb + k) / f - (L - 1) + (c - rr * L);
+                                                    y = 0.0f;
+                                                    if ((unsigned)aa < (unsigned)im.H && (unsigned)bb < (unsigned)im.W) {
+                                                        const Dat4<float> dv = dat_g[(size_t)aa * im.W + bb];
+                                                        int b = 0;
+                                                        y = dl_pixel_call(mu, xk, dv.c, dv.is2, dv.beta, &b);
+                                                        badL |= b ? 1u << k : 0u;
+                                                    }
                                                 }
                                             }
 #pragma unroll
