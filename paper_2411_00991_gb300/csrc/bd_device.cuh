@@ -263,6 +263,14 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, int x, 
         "l"(tmap), "r"(x), "r"(y), "r"(smem_u32(bar))
         : "memory");
 }
+// Before a block's first copy by a tensor map in global memory: the maps are
+// rewritten in place by host copies (a new plan, another handle's arena, the
+// serving loop's tables), which the descriptor reads of the tensormap proxy see
+// only after this acquire.
+__device__ __forceinline__ void tensormap_acquire(const void* tmap)
+{
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tmap) : "memory");
+}
 // Orders this thread's earlier generic-proxy accesses to global memory (and
 // those made visible to it by barriers and acquire fences) before its later
 // async-proxy (TMA) accesses.

@@ -182,6 +182,11 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sweep_rows(SweepArgs a)
     // have finished (kind 0, right: the run's classes but the last; 1: the
     // previous class row; 2: the previous sweep)
     const bool service = warp == nw - 1;
+    if (service && lane == 0) {
+        tensormap_acquire(tmap);
+        tensormap_acquire(tmap + 128);
+        if constexpr (!AUG) tensormap_acquire(tmap + 256);
+    }
     const uint32_t* nword = nullptr;
     int nkind = 0;
     if (lane < 8) {

@@ -626,6 +626,10 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
         for (int b = 0; b < 2; ++b)
             if ((stg_pend >> b) & 1u) stage_wait(b);
     };
+    if (SWIN && in_team && lt == 0) {   // the thread that issues the team's copies
+        const char* tm = reinterpret_cast<const char*>(ch.tmap);
+        for (int k = 0; k < 3; ++k) tensormap_acquire(tm + 128 * k);
+    }
     if (SANY) stage_issue(0);
     if (ahead && in_team && twarp == pwarp) {
         if constexpr (LEAN) {
