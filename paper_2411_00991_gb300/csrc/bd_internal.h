@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "bd_smem.h"
+
 namespace bd {
 
 constexpr int kMaxShapes = 4;       // patch shapes: full, right, bottom, corner
@@ -296,8 +298,20 @@ inline int refresh_blocks(int H, int W, int f)
     return refresh_small(H, W) ? ((W + 31) / 32) * ((H + 3) / 4) : ((W + 63) / 64) * ((H + 15) / 16);
 }
 
+// Makes fn's dynamic shared-memory limit on the current device at least bytes.
+inline cudaError_t raise_smem_limit(const void* fn, size_t bytes)
+{
+    static SmemLimits limits;
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return limits.raise(dev, fn, bytes, cudaSuccess, [](const void* f, size_t b) {
+        return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
+    });
+}
+
 // host launchers (defined in the .cu files)
-void launch_setup(const Image& im, const Image* d_im, const float* w, const float* g,
+cudaError_t launch_setup(const Image& im, const Image* d_im, const float* w, const float* g,
                   const float* o, const float* v, double gs, double os, double vs,
                   const double* psf_raw, double* b0_out, double* scratch, cudaStream_t st,
                   int64_t* launches);
@@ -309,7 +323,7 @@ template <typename T>
 // when out_index is null)
 // (with write_state on an augmented chain, the total is the log of the joint
 // density p(w, phi, rho) at the chain's photon counts)
-void launch_refresh(const Image& im, const Chain& ch, double* scratch, int write_state,
+cudaError_t launch_refresh(const Image& im, const Chain& ch, double* scratch, int write_state,
                     double* out_logpost, const int* out_index, int* err, cudaStream_t st, int64_t* launches);
 // out[k] = log k!, k < kLgamma
 void launch_lgamma(double* out, cudaStream_t st, int64_t* launches);

@@ -39,9 +39,6 @@
 // and 0.91; 2048 x 2048 L = 31 x 4 chains 189 and 97; six frames 128..768
 // x 4 chains 52 and 22; 64 x 64 L = 9 0.30 and 0.12; 150 x 150 on a twice finer
 // lattice 1.13 and 0.40.
-#include <map>
-#include <mutex>
-
 #include "bd_device.cuh"
 #include "bd_update.cuh"
 
@@ -803,18 +800,6 @@ const void* rows_fn(bool aug, bool fine, int vg, int threads)
                : fine ? rows_fn_of<false, true>(vg, threads) : rows_fn_of<false, false>(vg, threads);
 }
 
-cudaError_t rows_smem_limit(const void* fn, size_t smem)
-{
-    static std::map<const void*, size_t> limit;
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
-    size_t& cur = limit[fn];
-    if (cur >= smem) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) cur = smem;
-    return e;
-}
-
 }  // namespace
 
 cudaError_t launch_sweep_rows(const SweepArgs& a, int grid, int threads, size_t smem, cudaStream_t st)
@@ -822,7 +807,7 @@ cudaError_t launch_sweep_rows(const SweepArgs& a, int grid, int threads, size_t 
     SweepArgs args = a;
     void* kargs[] = {&args};
     const void* fn = rows_fn(a.aug != 0, a.fine != 0, a.row_vg, threads);
-    cudaError_t e = rows_smem_limit(fn, smem);
+    cudaError_t e = raise_smem_limit(fn, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -841,7 +826,7 @@ int rows_blocks_per_sm(bool aug, bool fine, int vg, int threads, size_t smem)
 {
     const void* fn = rows_fn(aug, fine, vg, threads);
     int n = 0;
-    if (rows_smem_limit(fn, smem) != cudaSuccess ||
+    if (raise_smem_limit(fn, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -11,8 +11,6 @@
 // not depend on the launch plan of the sweep kernel.
 #include <cmath>
 
-#include <atomic>
-#include <mutex>
 
 #include "bd_device.cuh"
 
@@ -202,7 +200,7 @@ __global__ void k_init_rho(int n, uint32_t seed_lo, uint32_t seed_hi, int chain,
     rho[m] = (T)(b0[0] * exp(0.1 * z));
 }
 
-void launch_setup(const Image& im, const Image* d_im, const float* w, const float* g, const float* o,
+cudaError_t launch_setup(const Image& im, const Image* d_im, const float* w, const float* g, const float* o,
                   const float* v, double gs, double os, double vs, const double* psf_raw, double* b0_out,
                   double* scratch, cudaStream_t st, int64_t* launches)
 {
@@ -229,14 +227,8 @@ void launch_setup(const Image& im, const Image* d_im, const float* w, const floa
                                       const_cast<float*>(im.tw32) + 2 * sh.tww_off);
         double* mag = scratch + nblk + 8;
         const size_t sm = 24 * (size_t)sh.ph * sh.pw;
-        static std::atomic<size_t> limit{46 * 1024};   // the dynamic shared-memory limit only grows (the static sums count too)
-        static std::mutex mu;
-        if (sm > limit.load()) {
-            std::lock_guard<std::mutex> lock(mu);
-            if (sm > limit.load() &&
-                cudaFuncSetAttribute(k_setup_alpha, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess)
-                limit.store(sm);
-        }
+        const cudaError_t e = raise_smem_limit((const void*)k_setup_alpha, sm);
+        if (e != cudaSuccess) return e;
         k_setup_alpha<<<1, kRedThreads, sm, st>>>(im.L, im.K64, sh.ph, sh.pw, im.ent_kl + sh.ent_off, sh.nhalf, mag,
                                                  const_cast<double*>(im.ent_wa64) + sh.ent_off,
                                                  const_cast<double*>(im.ent_m64) + sh.ent_off,
@@ -246,6 +238,7 @@ void launch_setup(const Image& im, const Image* d_im, const float* w, const floa
                                                  reinterpret_cast<const double2*>(im.tw64) + sh.tww_off);
         *launches += 3;
     }
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -457,7 +450,7 @@ __global__ void __launch_bounds__(kRedThreads) k_refresh_total(const double* par
 }
 
 template <typename T>
-void launch_refresh(const Image& im, const Chain& ch, double* scratch, int write_state, double* out_logpost,
+cudaError_t launch_refresh(const Image& im, const Chain& ch, double* scratch, int write_state, double* out_logpost,
                     const int* out_index, int* err, cudaStream_t st, int64_t* launches)
 {
     const int nblk = refresh_blocks(im.H, im.W, im.f);
@@ -470,35 +463,24 @@ void launch_refresh(const Image& im, const Chain& ch, double* scratch, int write
         const void* fn = small ? (const void*)k_refresh_mu<T, 32, 4, 1> : (const void*)k_refresh_mu<T, 64, 4, 4>;
         const int TC = (small ? 32 : 64) + im.L - 1, TR = (small ? 4 : 16) + im.L - 1;
         const size_t sm = 8 * (size_t)(((im.L * im.L + 1) & ~1) + TC * TR);
-        static std::atomic<size_t> lim[2] = {{48 * 1024 - 2048}, {48 * 1024 - 2048}};   // (the static sums count too)
-        static std::mutex mu_lim;
-        if (sm > lim[small].load()) {
-            std::lock_guard<std::mutex> lock(mu_lim);
-            if (sm > lim[small].load() &&
-                cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess)
-                lim[small].store(sm);
-        }
+        const cudaError_t e = raise_smem_limit(fn, sm);
+        if (e != cudaSuccess) return e;
         if (small) k_refresh_mu<T, 32, 4, 1><<<nblk, 128, sm, st>>>(im, ch, part_ll, write_state, err);
         else k_refresh_mu<T, 64, 4, 4><<<nblk, 256, sm, st>>>(im, ch, part_ll, write_state, err);
     }
     // the patch and its row transforms in shared memory (24 bytes per patch pixel)
     const size_t smem = 8 * (size_t)(((size_t)im.S * im.S + 1) / 2 * 2) + 16 * (size_t)im.S * im.S;
-    static std::atomic<size_t> limit{48 * 1024};   // the dynamic shared-memory limit only grows
-    static std::mutex mu;
-    if (smem > limit.load()) {
-        std::lock_guard<std::mutex> lock(mu);
-        if (smem > limit.load() &&
-            cudaFuncSetAttribute(k_refresh_spec<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
-            limit.store(smem);
-    }
+    const cudaError_t e = raise_smem_limit((const void*)k_refresh_spec<T>, smem);
+    if (e != cudaSuccess) return e;
     k_refresh_spec<T><<<im.n_patches, kRedThreads, smem, st>>>(im, ch, part_lp, write_state);
     k_refresh_total<<<1, kRedThreads, 0, st>>>(part_ll, nblk, part_lp, im.n_patches, out_logpost, out_index);
     *launches += 3;
+    return cudaGetLastError();
 }
-template void launch_refresh<float>(const Image&, const Chain&, double*, int, double*, const int*, int*, cudaStream_t,
-                                    int64_t*);
-template void launch_refresh<double>(const Image&, const Chain&, double*, int, double*, const int*, int*, cudaStream_t,
-                                     int64_t*);
+template cudaError_t launch_refresh<float>(const Image&, const Chain&, double*, int, double*, const int*, int*, cudaStream_t,
+                                           int64_t*);
+template cudaError_t launch_refresh<double>(const Image&, const Chain&, double*, int, double*, const int*, int*, cudaStream_t,
+                                            int64_t*);
 
 // ------------------------------------------------- photon-count draw -----
 __global__ void k_lgamma(double* out)
@@ -836,8 +818,7 @@ cudaError_t launch_quantiles(const void* samples, int64_t chain_stride, int n_ch
     int npow2 = 2;
     while (npow2 < n) npow2 <<= 1;
     const size_t smem = sizeof(double) * (size_t)npow2;
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_quantiles<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const cudaError_t e = raise_smem_limit((const void*)k_quantiles<T>, smem);
     if (e != cudaSuccess) return e;
     k_quantiles<T><<<(unsigned)npix, 256, smem, st>>>(reinterpret_cast<const T*>(samples), chain_stride, n_chains,
                                                       first, count, obj_pixels, Wo, crop_r, out_w, pix0, npow2, q,

@@ -33,10 +33,6 @@
 // mu, shared with the neighbouring tiles, is read from global memory (L2).
 #include <type_traits>
 
-#include <atomic>
-#include <map>
-#include <mutex>
-
 #include "bd_device.cuh"
 #include "bd_update.cuh"
 
@@ -1152,21 +1148,12 @@ const void* sweep_fn(bool res, bool aug, bool fine, bool solo, int stg, bool lea
     return res ? (const void*)k_sweep<T, true, false, false> : (const void*)k_sweep<T, false, false, false>;
 }
 
-// Raise a kernel form's dynamic shared-memory limit to at least smem.  The
-// limit is kept per kernel function (several form flags can name the same
-// function), and it only grows, so launches with smaller plans stay valid.
+// Raise a kernel form's dynamic shared-memory limit to at least smem (several
+// form flags can name the same function).
 template <typename T>
 cudaError_t ensure_smem_limit(bool res, bool aug, bool fine, bool solo, int stg, size_t smem, bool lean = false)
 {
-    static std::map<const void*, size_t> limit;
-    static std::mutex mu;
-    const void* fn = sweep_fn<T>(res, aug, fine, solo, stg, lean);
-    std::lock_guard<std::mutex> lock(mu);
-    size_t& cur = limit[fn];
-    if (cur >= smem) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) cur = smem;
-    return e;
+    return raise_smem_limit(sweep_fn<T>(res, aug, fine, solo, stg, lean), smem);
 }
 
 // Cooperative launch (all blocks co-resident, which the neighbour waits

@@ -896,9 +896,9 @@ bdecon_status refresh_chain(bdecon_handle* h, int ci, int write, double* out, co
 {
     const Chain& ch = h->chains[ci];
     const ProbHost& ph = h->probs[ch.img];
-    launch_refresh<T>(h->imgs[ch.img], ch, (double*)(h->arena + ph.o_scr), write, out, idx, h->d_err, h->st,
-                      &h->launches);
-    CK(h, cudaGetLastError());
+    const cudaError_t e = launch_refresh<T>(h->imgs[ch.img], ch, (double*)(h->arena + ph.o_scr), write, out, idx, h->d_err,
+                                            h->st, &h->launches);
+    if (e != cudaSuccess) return fail(h, BDECON_ERR_CUDA, "refresh launch: %s", cudaGetErrorString(e));
     return BDECON_OK;
 }
 
@@ -1191,8 +1191,9 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
         if (e != cudaSuccess) return bail(fail(h, BDECON_ERR_CUDA, "input upload: %s", cudaGetErrorString(e)));
         double* scr = (double*)(h->arena + ph.o_scr);
         double* b0 = h->d_out;
-        launch_setup(h->imgs[k], h->d_imgs + k, u_w, p.gain_map ? u_g : nullptr, p.offset_map ? u_o : nullptr,
-                     p.var_map ? u_v : nullptr, p.gain, p.offset, p.read_var, u_psf, b0, scr, h->st, &h->launches);
+        e = launch_setup(h->imgs[k], h->d_imgs + k, u_w, p.gain_map ? u_g : nullptr, p.offset_map ? u_o : nullptr,
+                         p.var_map ? u_v : nullptr, p.gain, p.offset, p.read_var, u_psf, b0, scr, h->st, &h->launches);
+        if (e != cudaSuccess) return bail(fail(h, BDECON_ERR_CUDA, "set-up launch: %s", cudaGetErrorString(e)));
         for (int c = 0; c < p.n_chains; ++c) {
             const Chain& ch = h->chains[ph.chain0 + c];
             if (h->precision == BDECON_FP32) launch_init_rho<float>(h->imgs[k], ch, b0, h->st, &h->launches);
