@@ -135,9 +135,14 @@ typedef struct {
 
 /* ------------------------------------------------------------- lifetime */
 
-/* Bytes of device workspace bdecon_create_in needs for these problems.  (In
- * double 112 bytes a camera pixel and chain of it hold likelihood records
- * that make the sweep faster; a workspace without them is accepted too.)    */
+/* Bytes of device workspace bdecon_create_in needs for these problems.  In
+ * double, 112 bytes a camera pixel and chain of it hold the marginal chains'
+ * likelihood records.  A workspace short of just those is accepted too, and so
+ * is a problem whose records the device (bdecon_create) or a server's budget
+ * does not hold: the records then lie in page-locked host memory.  Results are
+ * the same bit for bit; sweeps are slower (1.05x on a 64 x 64 frame, 1.2x to
+ * 1.6x on 250 x 203, 2.3x to 4.2x from 512 x 512 up).  bdecon_get_records
+ * tells.                                                                    */
 bdecon_status bdecon_workspace_size(const bdecon_problem* problems, int32_t n_problems,
                                     size_t* bytes);
 
@@ -255,6 +260,10 @@ bdecon_status bdecon_accept_log(bdecon_handle* h, int32_t p, int32_t c, uint8_t*
  * sweeps done.                                                              */
 bdecon_status bdecon_get_state(bdecon_handle* h, int32_t p, int32_t c, double* rho,
                                int64_t* sweeps);
+
+/* Where the double chains' likelihood records lie: 0 no records (float or
+ * augmented problems only), 1 device, 2 page-locked host memory.           */
+bdecon_status bdecon_get_records(const bdecon_handle* h, int32_t* where);
 
 /* Replace the object of chain c (all values > 0 and finite) and its sweep
  * counter, then refresh mu, spectra and log posterior in double.  The
@@ -403,7 +412,9 @@ bdecon_status bdecon_sweep_kernel_time(bdecon_handle* h, double* ms, int64_t* la
 typedef struct bdecon_server bdecon_server;
 
 typedef struct {
-    size_t mem_budget;         /* device bytes for the running jobs' workspaces     */
+    size_t mem_budget;         /* device bytes for the running jobs' workspaces (a double
+                                  job that fits only without its likelihood records keeps
+                                  them in page-locked host memory)                    */
     int32_t max_jobs;          /* jobs running at once, >= 1                         */
     int32_t segment_sweeps;    /* sweeps per shared segment, 1..64                  */
     int32_t precision;         /* bdecon_precision of every job                      */

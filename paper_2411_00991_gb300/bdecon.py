@@ -61,7 +61,8 @@ EXPORTS = ["bdecon_workspace_size", "bdecon_create", "bdecon_batch_create", "bde
            "bdecon_server_stop", "bdecon_set_grouping", "bdecon_autotune", "bdecon_set_graph",
            "bdecon_posterior_std", "bdecon_posterior_cv", "bdecon_get_samples", "bdecon_posterior_quantiles",
            "bdecon_get_steps", "bdecon_get_phi", "bdecon_set_staging", "bdecon_get_staging",
-           "bdecon_set_tuning_cache", "bdecon_set_lean", "bdecon_get_lean", "bdecon_get_form"]
+           "bdecon_set_tuning_cache", "bdecon_set_lean", "bdecon_get_lean", "bdecon_get_form",
+           "bdecon_get_records"]
 
 JOB_QUEUED, JOB_RUNNING, JOB_DONE, JOB_FAILED = 0, 1, 2, 3
 
@@ -111,6 +112,7 @@ def load(build_if_missing: bool = True):
         "bdecon_set_staging": [H, i32],
         "bdecon_get_staging": [H, i32, C.POINTER(i32)],
         "bdecon_set_lean": [H, i32],
+        "bdecon_get_records": [H, C.POINTER(i32)],
         "bdecon_get_lean": [H, i32, C.POINTER(i32)],
         "bdecon_get_form": [H, i32, C.POINTER(i32), C.POINTER(i32), C.POINTER(i32), C.POINTER(i32)],
         "bdecon_launch_count": [H, C.POINTER(i64)],
@@ -427,6 +429,12 @@ class Sampler:
         """1 when problem p's launch group runs the lean kernel form, else 0."""
         v = C.c_int32()
         self._ck(self.L.bdecon_get_lean(self.h, p, C.byref(v)))
+        return int(v.value)
+
+    def records(self) -> int:
+        """Where the double chains' likelihood records lie: 0 none, 1 device, 2 page-locked host memory."""
+        v = C.c_int32()
+        self._ck(self.L.bdecon_get_records(self.h, C.byref(v)))
         return int(v.value)
 
     def form(self, p: int = 0):

@@ -63,15 +63,15 @@ __device__ __forceinline__ bool win_cell(const Image& im, int i, int j, int k, i
            (unsigned)q < (unsigned)Le;
 }
 
-// Likelihood part of one update for one team thread: fetches the expected
-// image (and, for float sweeps, the cached cumulants) of its window pixels
+// Likelihood part of one update for one team thread of a float marginal chain:
+// fetches the expected image and the cached cumulants of its window pixels
 // in one batch, sums their Eq. 6 changes, and leaves the warp's partial sum
 // and bad flag in out[0..1].  muv keeps the fetched expected image values.
 // Fetch the first batch of a thread's window values (expected image and
 // cached cumulants) so the loads are in flight while other work proceeds.
-template <typename T, bool CUM, bool FINE, int NPX = kMaxPx>
-__device__ __forceinline__ void window_fetch(const T* mu_g, const float4* cum_g, const float2* cum2_g,
-                                             const Image& im, int i, int j, int lt, T (&muv)[NPX],
+template <bool FINE, int NPX = kMaxPx>
+__device__ __forceinline__ void window_fetch(const float* mu_g, const float4* cum_g, const float2* cum2_g,
+                                             const Image& im, int i, int j, int lt, float (&muv)[NPX],
                                              float4 (&cq)[NPX], float2 (&cq2)[NPX], int k0)
 {
     const int NT = im.team;
@@ -98,26 +98,24 @@ __device__ __forceinline__ void window_fetch(const T* mu_g, const float4* cum_g,
                 ++kr;
             }
         }
-        muv[jj] = in ? __ldcg(mu_g + (size_t)aa * im.mu_pitch + bb) : (T)-1;
-        if (CUM) {
-            cq[jj] = in ? __ldcg(cum_g + (size_t)aa * im.mu_pitch + bb) : make_float4(0, 0, 0, 0);
-            cq2[jj] = in ? __ldcg(cum2_g + (size_t)aa * im.mu_pitch + bb) : make_float2(0, 0);
-        }
+        muv[jj] = in ? __ldcg(mu_g + (size_t)aa * im.mu_pitch + bb) : -1.0f;
+        cq[jj] = in ? __ldcg(cum_g + (size_t)aa * im.mu_pitch + bb) : make_float4(0, 0, 0, 0);
+        cq2[jj] = in ? __ldcg(cum2_g + (size_t)aa * im.mu_pitch + bb) : make_float2(0, 0);
     }
 }
 
-template <typename T, bool RES, bool CUM, bool FINE, int NPX = kMaxPx>
-__device__ __forceinline__ void lik_partial(const T* mu_g, const float4* cum_g, const float2* cum2_g, const Dat4<T>* dat_s,
-                                            const Dat4<T>* dat_g, const T* Ks, const Image& im, int i, int j,
-                                            int a_lo, int b_lo, int rw, int lt, int NT, T delta, T (&muv)[NPX],
-                                            T* out, int lane, float4 (&cq)[NPX], float2 (&cq2)[NPX],
-                                            bool prefetched)
+template <bool RES, bool FINE, int NPX = kMaxPx>
+__device__ __forceinline__ void lik_partial(const float* mu_g, const float4* cum_g, const float2* cum2_g,
+                                            const Dat4<float>* dat_s, const Dat4<float>* dat_g, const float* Ks,
+                                            const Image& im, int i, int j, int a_lo, int b_lo, int rw, int lt, int NT,
+                                            float delta, float (&muv)[NPX], float* out, int lane, float4 (&cq)[NPX],
+                                            float2 (&cq2)[NPX], bool prefetched)
 {
     const int W = im.W, LL = FINE ? im.Lc * im.Lc : im.L * im.L;
-    T accL = 0;
+    float accL = 0;
     bool badL = false;
     for (int k0 = lt; k0 < LL; k0 += NT * NPX) {
-        if (!(prefetched && k0 == lt)) window_fetch<T, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, im, i, j, lt, muv, cq, cq2, k0);
+        if (!(prefetched && k0 == lt)) window_fetch<FINE, NPX>(mu_g, cum_g, cum2_g, im, i, j, lt, muv, cq, cq2, k0);
 #pragma unroll
         for (int jj = 0; jj < NPX; ++jj) {
             const int k = k0 + jj * NT;
@@ -125,26 +123,19 @@ __device__ __forceinline__ void lik_partial(const T* mu_g, const float4* cum_g, 
             // inside, -1 outside), so the geometry is needed only to read the
             // cell's data on the exact path; the finer lattice needs its PSF index
             int aa = 0, bb = 0, kw = k;
-            const bool in = FINE ? win_cell<FINE>(im, i, j, k, aa, bb, kw) : muv[jj] != (T)-1;
+            const bool in = FINE ? win_cell<FINE>(im, i, j, k, aa, bb, kw) : muv[jj] != -1.0f;
             if (in) {
-                const T xk = mul_rn(delta, Ks[kw]);
-                if (CUM) {
-                    const float d = (float)xk * Prec<float>::rcp((float)muv[jj]);
-                    if (fabsf(d) <= kCumEval) {
-                        accL += (T)cgf_delta((float)xk, log1p_cum(d), cq[jj], cq2[jj]);
-                        continue;
-                    }
+                const float xk = mul_rn(delta, Ks[kw]);
+                const float d = xk * Prec<float>::rcp(muv[jj]);
+                if (fabsf(d) <= kCumEval) {
+                    accL += cgf_delta(xk, log1p_cum(d), cq[jj], cq2[jj]);
+                    continue;
                 }
                 if (!FINE) win_cell<FINE>(im, i, j, k, aa, bb, kw);
-                const Dat4<T> dv = RES ? dat_s[(aa - a_lo) * rw + (bb - b_lo)] : dat_g[(size_t)aa * W + bb];
-                if (CUM) {
-                    int b = 0;
-                    accL += (T)dl_pixel_call((float)muv[jj], (float)xk, (float)dv.c, (float)dv.is2, (float)dv.beta,
-                                             &b);
-                    badL = badL || b;
-                } else {
-                    accL += dl_pixel<T>(muv[jj], xk, dv.c, dv.is2, dv.beta, badL);
-                }
+                const Dat4<float> dv = RES ? dat_s[(aa - a_lo) * rw + (bb - b_lo)] : dat_g[(size_t)aa * W + bb];
+                int b = 0;
+                accL += dl_pixel_call(muv[jj], xk, dv.c, dv.is2, dv.beta, &b);
+                badL = badL || b;
             }
         }
     }
@@ -152,7 +143,7 @@ __device__ __forceinline__ void lik_partial(const T* mu_g, const float4* cum_g, 
     const bool wb = __any_sync(0xffffffffu, badL);
     if (lane == 0) {
         out[0] = accL;
-        out[1] = wb ? (T)1 : (T)0;
+        out[1] = wb ? 1.0f : 0.0f;
     }
 }
 
@@ -315,7 +306,7 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
     // augmented sampler (AUG) scores windows from the photon counts instead
     constexpr bool CUM = std::is_same<T, float>::value && !AUG;
     constexpr bool DEC1 = std::is_same<T, double>::value;          // one warp of a team decides
-    constexpr bool C64 = std::is_same<T, double>::value && !AUG;   // cumulant records, where the chain has them
+    constexpr bool C64 = std::is_same<T, double>::value && !AUG;   // cumulant records
     static_assert(STG == 0 || (std::is_same<T, float>::value && !AUG && !FINE && !SOLO), "staging: float marginal camera grid");
     constexpr bool SANY = STG != 0;                          // staging
     constexpr bool SWIN = STG == 1;                          // the window is staged
@@ -769,7 +760,7 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
             // latency overlaps the arithmetic below
             if (active && !SWIN) {
                 if constexpr (AUG) window_fetch_aug<T, FINE, NPX>(mu_g, phi_g, im, i, j, muv, phv, lt);
-                else if (!C64 || ch.cum64 == nullptr) window_fetch<T, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, im, i, j, lt, muv, cq, cq2, lt);
+                else if constexpr (CUM) window_fetch<FINE, NPX>(mu_g, cum_g, cum2_g, im, i, j, lt, muv, cq, cq2, lt);
             }
             // a2 + a4: proposal and prior change (own tile state only)
             if (active) {
@@ -814,19 +805,12 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
                 else if constexpr (SWIN)
                     lik_partial_staged<RES>(wmu, wcum, wcum2, BW, wdx, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt,
                                             NT, delta, pr2 + twarp * 4, lane);
-                else {
-                    bool done = false;
-                    if constexpr (C64) {
-                        if (ch.cum64 != nullptr) {
-                            lik_partial64<RES, FINE>(mu_g, ch.cum64, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT, delta,
-                                                     pr2 + twarp * 4, lane);
-                            done = true;
-                        }
-                    }
-                    if (!done)
-                        lik_partial<T, RES, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt,
-                                                            NT, delta, muv, pr2 + twarp * 4, lane, cq, cq2, true);
-                }
+                else if constexpr (C64)
+                    lik_partial64<RES, FINE>(mu_g, ch.cum64, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT, delta,
+                                             pr2 + twarp * 4, lane);
+                else
+                    lik_partial<RES, FINE, NPX>(mu_g, cum_g, cum2_g, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT, delta,
+                                                muv, pr2 + twarp * 4, lane, cq, cq2, true);
             }
             // a5: Metropolis-Hastings decision with the Hastings term of the log-space
             // walk, taken from the round's partial sums as soon as every warp of the
@@ -952,18 +936,12 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
                         stage_wait(sb);
                         lik_partial_staged<RES>(wmu, wcum, wcum2, BW, wdx, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw,
                                                 lt, NT, delta, pr2 + twarp * 4, lane);
+                    } else if constexpr (C64) {
+                        lik_partial64<RES, FINE>(mu_g, ch.cum64, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT, delta,
+                                                 pr2 + twarp * 4, lane);
                     } else {
-                        bool done = false;
-                        if constexpr (C64) {
-                            if (ch.cum64 != nullptr) {
-                                lik_partial64<RES, FINE>(mu_g, ch.cum64, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT,
-                                                         delta, pr2 + twarp * 4, lane);
-                                done = true;
-                            }
-                        }
-                        if (!done)
-                            lik_partial<T, RES, CUM, FINE, NPX>(mu_g, cum_g, cum2_g, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw,
-                                                                lt, NT, delta, muv, pr2 + twarp * 4, lane, cq, cq2, false);
+                        lik_partial<RES, FINE, NPX>(mu_g, cum_g, cum2_g, dat_s, dat_g, Ks, im, i, j, a_lo, b_lo, rw, lt, NT,
+                                                    delta, muv, pr2 + twarp * 4, lane, cq, cq2, false);
                     }
                 }
                 __syncthreads();
@@ -990,18 +968,16 @@ __global__ void __launch_bounds__(256, std::is_same<T, float>::value ? (LEAN ? 4
                                 // (unchanged since)
                                 const size_t idx = (size_t)aa * im.mu_pitch + bb;
                                 const int widx = (k / L) * BW + wdx + (k - (k / L) * L);
-                                const T old = SWIN ? (T)wmu[widx] : one_batch && !(C64 && ch.cum64 != nullptr) ? muv[jj] : __ldcg(mu_g + idx);
+                                const T old = SWIN ? (T)wmu[widx] : one_batch && !C64 ? muv[jj] : __ldcg(mu_g + idx);
                                 const T xk = mul_rn(delta, Ks[kw]);
                                 const T nmu = add_rn(old, xk);
                                 __stcg(mu_g + idx, nmu);
                                 if constexpr (C64) {
-                                    if (ch.cum64 != nullptr) {
-                                        double* rec = ch.cum64 + kCum64 * idx;
-                                        if (!cum64_shift(nmu, xk, rec)) {
-                                            const Dat4<T> dv =
-                                                RES ? dat_s[(aa - a_lo) * rw + (bb - b_lo)] : dat_g[(size_t)aa * W + bb];
-                                            photon_record64(nmu, dv.c, dv.is2, dv.beta, rec);
-                                        }
+                                    double* rec = ch.cum64 + kCum64 * idx;
+                                    if (!cum64_shift(nmu, xk, rec)) {
+                                        const Dat4<T> dv =
+                                            RES ? dat_s[(aa - a_lo) * rw + (bb - b_lo)] : dat_g[(size_t)aa * W + bb];
+                                        photon_record64(nmu, dv.c, dv.is2, dv.beta, rec);
                                     }
                                 }
                                 if (CUM) {
@@ -1259,7 +1235,7 @@ __global__ void __launch_bounds__(256) k_delta(const Image* imp, const Chain* ch
                 }
                 if constexpr (std::is_same<T, double>::value) {
                     double y;
-                    if (ch.cum64 != nullptr && cgf_delta64(xk, ch.cum64 + kCum64 * idx, y)) {
+                    if (cgf_delta64(xk, ch.cum64 + kCum64 * idx, y)) {
                         accL += y;
                         continue;
                     }

@@ -7,7 +7,9 @@
 #include <condition_variable>
 #include <deque>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <thread>
 #include <cstdarg>
 #include <cstdio>
@@ -114,6 +116,8 @@ struct bdecon_handle {
     char* arena = nullptr;
     size_t arena_bytes = 0;
     bool own_arena = false;
+    char* host_rec = nullptr;       // the double chains' records in page-locked host memory, where the arena has none
+    size_t host_rec_bytes = 0;
     size_t o_imgs = 0, o_chains = 0, o_err = 0, o_out = 0, o_scr = 0, o_up = 0;
     size_t up_bytes = 0;
     Image* d_imgs = nullptr;
@@ -814,13 +818,13 @@ bool encode_stage_maps(const ProbHost& ph, const Chain& ch, CUtensorMap out[3])
     return true;
 }
 
-// Device arena layout.  records: with the double chains' cumulant records
-// (112 bytes a camera pixel); without them the double sweep evaluates the
-// exact photon sums, and the arena is the smallest that works.
+// Device arena layout.  records: the double chains' cumulant records (112
+// bytes a camera pixel) in the arena, at o_cum64; else o_cum64 is their offset
+// in host memory, host_rec_bytes of it.
 size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainHost>& chh, int prec, int max_sweeps,
               bool records = true)
 {
-    Alloc A;
+    Alloc A, R;
     const size_t ts = prec == BDECON_FP32 ? 4 : 8;
     size_t up = 0;
     size_t scr_max = 0;
@@ -863,7 +867,8 @@ size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainH
             const bool aug = (ph.p.flags & BDECON_FLAG_AUGMENTED) != 0;
             x.o_cum = prec == BDECON_FP32 && !aug ? A.take(16 * (size_t)ph.H * ph.pitch) : 0;
             x.o_cum2 = prec == BDECON_FP32 && !aug ? A.take(8 * (size_t)ph.H * ph.pitch) : 0;
-            x.o_cum64 = prec == BDECON_FP64 && !aug && records ? A.take(8 * (size_t)kCum64 * ph.H * ph.pitch) : 0;
+            const size_t rec = prec == BDECON_FP64 && !aug ? 8 * (size_t)kCum64 * ph.H * ph.pitch : 0;
+            x.o_cum64 = !rec ? 0 : records ? A.take(rec) : R.take(rec);
             x.o_phi = aug ? A.take(ts * (size_t)ph.H * ph.pitch) : 0;
             x.o_tpart = A.take(8 * (size_t)kMaxSlots * ph.n_patches);
             x.o_acc = A.take(8 * (size_t)max_sweeps);
@@ -885,6 +890,7 @@ size_t layout(bdecon_handle* h, std::vector<ProbHost>& probs, std::vector<ChainH
     h->o_out = A.take(64);
     h->up_bytes = up;
     h->o_up = A.take(up);
+    h->host_rec_bytes = R.off;
     (void)scr_max;
     return align_up(A.off, 256);
 }
@@ -1023,6 +1029,7 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
     auto bail = [&](bdecon_status s) {
         std::string m = h->err;
         if (h->own_arena && h->arena) cudaFree(h->arena);
+        if (h->host_rec) cudaFreeHost(h->host_rec);
         delete h;
         g_err = m;
         return s;
@@ -1032,7 +1039,10 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (!coop) return bail(fail(h, BDECON_ERR_CUDA, "device does not support cooperative launches"));
-    // (the cumulant records of double chains are left out where memory is short)
+    // The double chains' records go to page-locked host memory where the caller's
+    // workspace, the device or a server's budget does not hold them: a chain's last
+    // digits depend on how its likelihood changes are summed, so every chain of a
+    // problem uses its records, wherever they fit.
     size_t need = layout(h, h->probs, h->chh, h->precision, h->max_sweeps, records);
     if (ws) {
         if (ws_bytes < need && records) need = layout(h, h->probs, h->chh, h->precision, h->max_sweeps, false);
@@ -1056,6 +1066,14 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
         h->own_arena = true;
     }
     h->arena_bytes = need;
+    if (h->host_rec_bytes) {
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, h->host_rec_bytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            return bail(fail(h, BDECON_ERR_NOMEM, "%zu bytes of page-locked host memory for likelihood records", h->host_rec_bytes));
+        }
+        h->host_rec = (char*)p;
+    }
     if (cudaMemsetAsync(h->arena, 0, need, h->st) != cudaSuccess) return bail(fail(h, BDECON_ERR_CUDA, "memset"));
     h->d_imgs = (Image*)(h->arena + h->o_imgs);
     h->d_chains = (Chain*)(h->arena + h->o_chains);
@@ -1112,7 +1130,8 @@ bdecon_status create_impl(const bdecon_problem* ps, int n, void* stream, void* w
             ch.rho = A + x.o_rho; ch.mu = A + x.o_mu; ch.spec = A + x.o_spec;
             ch.cum = x.o_cum ? (float4*)(A + x.o_cum) : nullptr;
             ch.cum2 = x.o_cum2 ? (float2*)(A + x.o_cum2) : nullptr;
-            ch.cum64 = x.o_cum64 ? (double*)(A + x.o_cum64) : nullptr;
+            const bool rec = h->precision == BDECON_FP64 && !(ph.p.flags & BDECON_FLAG_AUGMENTED);
+            ch.cum64 = rec ? (double*)((h->host_rec ? h->host_rec : A) + x.o_cum64) : nullptr;
             ch.rho_sum = (double*)(A + ph.o_sum) + c * nobj;
             ch.rho_sq = ph.o_sq ? (double*)(A + ph.o_sq) + c * nobj : nullptr;
             ch.trace_part = (double*)(A + x.o_tpart);
@@ -1512,6 +1531,7 @@ void bdecon_destroy(bdecon_handle* h)
     if (h->cap_st) cudaStreamDestroy(h->cap_st);
     for (cudaEvent_t ev : h->ev_pool) cudaEventDestroy(ev);
     if (h->own_arena && h->arena) cudaFree(h->arena);
+    if (h->host_rec) cudaFreeHost(h->host_rec);
     delete h;
 }
 
@@ -1977,6 +1997,15 @@ bdecon_status bdecon_get_lean(bdecon_handle* h, int32_t p, int32_t* lean)
     return BDECON_OK;
 }
 
+bdecon_status bdecon_get_records(const bdecon_handle* h, int32_t* where)
+{
+    if (!h || !where) return fail(nullptr, BDECON_ERR_INVALID, "bad arguments");
+    *where = 0;
+    for (const Chain& ch : h->chains)
+        if (ch.cum64) *where = h->host_rec ? 2 : 1;
+    return BDECON_OK;
+}
+
 bdecon_status bdecon_get_form(bdecon_handle* h, int32_t p, int32_t* run, int32_t* per_team, int32_t* resident,
                               int32_t* one_team)
 {
@@ -2032,6 +2061,13 @@ bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* o
         cudaGetLastError();
         return fail(h, BDECON_ERR_NOMEM, "autotune needs a %zu-byte copy of the workspace", h->arena_bytes);
     }
+    // (and the records, where they lie in host memory: the stream is idle)
+    const std::unique_ptr<char[]> rec_snap(h->host_rec ? new (std::nothrow) char[h->host_rec_bytes] : nullptr);
+    if (h->host_rec && !rec_snap) {
+        cudaFree(snap);
+        return fail(h, BDECON_ERR_NOMEM, "autotune needs a %zu-byte copy of the likelihood records", h->host_rec_bytes);
+    }
+    if (rec_snap) std::memcpy(rec_snap.get(), h->host_rec, h->host_rec_bytes);
     CK(h, cudaMemcpyAsync(snap, h->arena, h->arena_bytes, cudaMemcpyDeviceToDevice, h->st));
     const int64_t sweeps0 = h->sweeps;
     std::vector<int64_t> nsum0;
@@ -2039,6 +2075,7 @@ bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* o
     auto restore = [&]() -> bdecon_status {
         CK(h, cudaMemcpyAsync(h->arena, snap, h->arena_bytes, cudaMemcpyDeviceToDevice, h->st));
         CK(h, cudaStreamSynchronize(h->st));
+        if (rec_snap) std::memcpy(h->host_rec, rec_snap.get(), h->host_rec_bytes);
         h->sweeps = sweeps0;
         for (size_t k = 0; k < h->probs.size(); ++k) h->probs[k].n_sum = nsum0[k];
         return BDECON_OK;
@@ -2239,7 +2276,7 @@ struct SrvJob {
     int state = BDECON_JOB_QUEUED;
     double t_submit = 0, t_start = 0, t_done = 0;
     size_t mem = 0;
-    bool records = true;                // with the double chains' cumulant records (where the budget holds them)
+    bool records = true;                // the double chains' records in device memory (where the budget holds them)
     bdecon_handle* h = nullptr;
     std::vector<double> mean;
     std::string err;
