@@ -70,6 +70,7 @@ struct Group {
     size_t smem = 0;
     int resident = 1;
     bool streamed = false;             // plan with tile state in global memory even if it fits in shared
+    bool user_stream = false;          // streamed set by the autotuner: the planner does not choose it
     bool aug = false;                  // photon-count augmented problems (their own kernel form)
     bool fine = false;                 // object lattices finer than the camera (their own kernel form)
     bool solo = false;                 // every block: one patch, one team (a kernel form of its own)
@@ -695,7 +696,7 @@ bool plan_items(int precision, int sms, std::vector<PlanItem*>& items, Group& g,
         }
         return plan_rows(precision, sms, items, g);
     }
-    if (precision == BDECON_FP64 && !g.streamed && g.no_stage) {
+    if (precision == BDECON_FP64 && !g.streamed && !g.user_stream && g.no_stage) {
         auto cost = [&](const Group& q) {
             int area = 1;
             for (const PlanItem* it : items)
@@ -948,6 +949,7 @@ void apply_choice(Group& g, const TuneChoice& c)
     g.user_warps = !c.rows;
     if (!c.rows) g.warps = c.warps;
     g.streamed = c.streamed;
+    g.user_stream = !c.rows;
     g.no_stage = !c.staged;
     g.user_stage = true;
     g.user_lean = c.rows ? -2 : c.lean ? 1 : 0;
@@ -2120,6 +2122,7 @@ bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* o
                         g.warps = w;
                         g.user_warps = true;
                         g.streamed = streamed != 0;
+                        g.user_stream = true;
                         g.no_stage = st == 0;
                         g.user_stage = true;
                         g.user_lean = ln;
@@ -2155,6 +2158,7 @@ bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* o
                     g.warps = w;
                     g.user_warps = true;
                     g.streamed = streamed != 0;
+                    g.user_stream = true;
                     g.no_stage = st == 0;
                     g.user_stage = true;
                     if (make_plan(h) != BDECON_OK) continue;
