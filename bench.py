@@ -349,7 +349,7 @@ def leg_widefield512(bd, stream, torch, dev, peaks, flush, checks, steps=3, swee
     nt = photon_terms(prob, s.get_mu())
     upd_launch = Ho * Wo * sweeps
     rf, bw = roofline(flops_per_update(prob.L, prob.S, nt) * upd_launch, kms, nl, upd_launch, dev, peaks,
-                      "k_sweep<float> one-team form")
+                      "k_sweep_rows (row-run form)")
     rho, t = s.get_state()
     checks.append(dict(leg="widefield_512", what=f"float chain, trace after sweep {t}", prob=prob, rho=rho,
                        trace=float(s.trace()[-1])))
@@ -405,7 +405,7 @@ def leg_lowsnr2048(bd, stream, torch, dev, peaks, checks):
     kms, nl = kernel_time(s, 2)
     nt = photon_terms(prob, s.get_mu(0, 0))
     out["roofline"], out["bw_roofline"] = roofline(flops_per_update(prob.L, prob.S, nt) * upd * 2, kms, nl,
-                                                   upd * 2, dev, peaks, "k_sweep<float>")
+                                                   upd * 2, dev, peaks, "k_sweep_rows (row-run form)")
     out["plan"] = s.get_plan()
     out["fp32"] = {"value": upd * 5 / (ms / 1e3), "unit": "pixel-updates/s", "ms_per_sweep": ms / 5}
     rho, t = s.get_state(0, 0)
@@ -521,7 +521,7 @@ def run_ours(args):
     nts = [photon_terms(q, s.get_mu(p, 0)) for p, q in enumerate(probs)]
     flops = S * sum((q.H + 2 * q.R) * (q.W + 2 * q.R) * q.n_chains * flops_per_update(q.L, q.S, nt)
                     for q, nt in zip(probs, nts))
-    rf, bw = roofline(flops, kms, nl, upd_sweep * S, dev, peaks, "k_sweep<float> (batched launch groups)")
+    rf, bw = roofline(flops, kms, nl, upd_sweep * S, dev, peaks, "k_sweep_rows (row-run form, batched launch groups)")
     checks = []
     order = np.argsort([q.H for q in probs])
     for p in (int(order[0]), int(order[len(order) // 2]), int(order[-1])):

@@ -316,20 +316,21 @@ bdecon_status bdecon_set_graph(bdecon_handle* h, int32_t enable);
 bdecon_status bdecon_set_grouping(bdecon_handle* h, int32_t one_launch);
 
 /* Autotuner: times trial segments of trial_sweeps sweeps (1..64) for each
- * launch shape -- per-group launches with 1x/2x/4x the team's warps, tile
- * state resident in shared memory or streamed from global, each group tuned
- * on its own; and the same shapes as one launch over every problem -- keeps
- * the fastest, and restores the chains exactly (a device copy of the whole
- * workspace is taken first: BDECON_ERR_NOMEM if it does not fit).  Tiles
- * become automatic.  Outputs (optional): the grouping chosen and the
+ * launch shape -- the row-run form where it applies; per-group class-by-class
+ * launches with 1x/2x/4x the team's warps, tile state resident in shared
+ * memory or streamed from global, each group tuned on its own; and the same
+ * shapes as one launch over every problem -- keeps the fastest, and restores
+ * the chains exactly (a copy of the whole workspace is taken first, on the
+ * device, and of records in host memory there: BDECON_ERR_NOMEM if one does
+ * not fit).  Tiles become automatic.  Outputs (optional): the grouping chosen and the
  * measured device milliseconds per sweep.  Synchronous.                   */
 bdecon_status bdecon_autotune(bdecon_handle* h, int32_t trial_sweeps, int32_t* one_launch,
                               double* ms_per_sweep);
 
 /* Tuning cache (process-wide; no counterpart in the paper, which describes
  * no implementation).  Each successful bdecon_autotune stores its choices
- * (grouping; per group: warps per block, resident or streamed tile state,
- * window staging) keyed by the device, the precision, the handle's staging
+ * (grouping; per group: row-run or class-by-class form, warps per block,
+ * resident or streamed tile state, window staging) keyed by the device, the precision, the handle's staging
  * setting and every problem's frame size, PSF side, stride, lattice factor,
  * chain count, sampler and update team, in order.  A handle created later
  * for the same key (bdecon_create, _batch_create, _create_in) starts with
@@ -358,14 +359,15 @@ bdecon_status bdecon_get_staging(bdecon_handle* h, int32_t p, int32_t* staged);
  * grid, unstaged plans other than the one-patch one-team form): each update
  * thread holds half as many window cells in flight (the window of Eq. 6 over
  * the PSF support, Fig. 5d) and the kernel is built for 64 registers a
- * thread, so more blocks are resident per SM.  mode -1 (the default): used
- * for PSF windows of more than 256 pixels (side 17 and up; measured faster
- * there, slower for smaller windows); 0: never; 1: wherever eligible.
- * bdecon_autotune tries both.  Results do not change.
- * With -1 float problems run, where it applies, the row-run form, which
- * scores runs of classes at once; 0 and 1 keep them in the class-by-class
- * forms.  bdecon_get_lean reports whether problem p's launch group runs the
- * lean form.                                                               */
+ * thread, so more blocks are resident per SM.  mode -1 (the default): float
+ * problems run the row-run form, which scores runs of classes at once, where
+ * it applies; where it does not (given block warps, staging, one launch over
+ * several PSF sides, strides below 3), the lean form for PSF windows of more
+ * than 256 pixels (side 17 and up; measured faster there, slower for smaller
+ * windows).  0 and 1 keep to the class-by-class forms, never or wherever
+ * eligible in the lean one.  bdecon_autotune tries all of them.  Results do
+ * not change.  bdecon_get_lean reports whether problem p's launch group runs
+ * the lean form, bdecon_get_form which other.                              */
 bdecon_status bdecon_set_lean(bdecon_handle* h, int32_t mode);
 bdecon_status bdecon_get_lean(bdecon_handle* h, int32_t p, int32_t* lean);
 

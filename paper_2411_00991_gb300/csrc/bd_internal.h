@@ -289,8 +289,15 @@ __host__ __device__ inline RowsSmem rows_smem(int L, int Le, int f, int V, int G
     return p;
 }
 
-// Blocks of the expected-image refresh: tiles of 32 x 4 camera pixels while
-// those leave SMs free, else of 64 x 16; a finer lattice takes 256 pixels a block.
+// Blocks of the expected-image refresh: tiles of 32 x 4 camera pixels up to 512
+// x 512, else of 64 x 16; a finer lattice takes 256 pixels a block.  us of a log
+// posterior, small and large tiles: 256 x 256 L = 9 113, 150, L = 31 240, 390; 512
+// x 512 L = 17 355, 384; 724 x 724 L = 17 658, 716; 1024 x 1024 L = 17 1229,
+// 1238; 1448 x 1448 L = 17 2438, 2426; 2048 x 2048 L = 31 9788, 9614.  The sides
+// are equal near 1400 x 1400.  The line was drawn lower before these were
+// measured and is kept, at 1 to 14% of a refresh between the two sizes, because it
+// also fixes the order in which a frame's log posterior is summed: moving it would
+// change the last digits of traces.
 inline bool refresh_small(int H, int W) { return (int64_t)H * W <= 256 * 1024; }
 inline int refresh_blocks(int H, int W, int f)
 {

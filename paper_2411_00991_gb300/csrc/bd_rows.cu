@@ -1,4 +1,5 @@
-// bd_rows.cu -- row-run form of the sweep kernel (float, camera grid).
+// bd_rows.cu -- row-run form of the sweep kernel (float: marginal on any object
+// lattice, augmented on the camera grid).
 //
 // The classes of a sweep are taken S at a time, one class row u at a time:
 // within a row the offsets v = 0..S-1 follow each other, and a block scores a

@@ -798,8 +798,8 @@ cudaError_t launch_quantiles(const void* samples, int64_t chain_stride, int n_ch
                              int64_t obj_pixels, int Wo, int crop_r, int out_w, int64_t pix0, int64_t npix,
                              const double* q, int nq, double* out, cudaStream_t st, int64_t* launches)
 {
-    // warp form while the block's values fit its static shared memory (47.5 KB):
-    // up to 256 values a pixel in float, 128 in double
+    // warp form while the block's values fit static shared memory (33 KB at 256
+    // values a pixel in float and 128 in double; twice as many would pass 48 KB)
     const int n = count * n_chains;
     const unsigned wb = (unsigned)((npix + kQuantPix - 1) / kQuantPix);
     const T* sp = reinterpret_cast<const T*>(samples);

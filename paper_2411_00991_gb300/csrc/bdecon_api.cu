@@ -684,7 +684,9 @@ bool plan_items(int precision, int sms, std::vector<PlanItem*>& items, Group& g,
         // against 0.63, 300 x 300 L = 9 x 2 chains 0.65 against 0.75; with three
         // warps or more teams a block, or tiles of several patches, the row runs
         // are ahead (512 x 512 L = 17 1.38 against 1.27, 256 x 256 L = 9 0.39
-        // against 0.28).
+        // against 0.28).  The forms are compared as they are: the one-team form's
+        // count step evaluates two double lgamma per pixel, the row runs' reads a
+        // table, so the line would move with that step.
         bool one = g.aug && g.threads <= 64;
         for (const PlanItem* it : items) one = one && it->tpi == 1 && it->tpj == 1 && g.threads == it->team;
         if (!one) return true;
