@@ -397,6 +397,12 @@ __device__ __forceinline__ int photon_mode(float muf, float cf, float isf)
     return __float2int_rn(phs);
 }
 
+// Most terms of a photon sum on either side of the mode estimate p0: the
+// photon posterior's standard deviation is at most sqrt(mu), so 4096 terms reach
+// 8.5 of them (2^-56 of the sum) up to p0 = 230 000, and p0 terms beyond.  The
+// sums normally end far sooner, at their smallest term that counts.
+__device__ __forceinline__ int phi_terms(int p0) { return max(4096, p0 + 1); }
+
 // Reciprocals 1/k of photon counts, correctly rounded (a table instead of a
 // double divide per photon term).
 constexpr int kRcpCount = 1024;
@@ -461,7 +467,8 @@ __device__ __forceinline__ T dl_pixel(T mu, T x, T c, T is2, T beta, bool& bad)
         T mg = mg0;
         T t = (T)1, e = (T)0;
         T fphi = fp0;
-        for (int it = 0; it < 2048; ++it) {
+        const int passes = phi_terms(p0) / 2;
+        for (int it = 0; it < passes; ++it) {
             T r1, r2;
             if constexpr (sizeof(T) == 8) {
                 r1 = rcp_count(p0 + 2 * it + 1);
@@ -584,7 +591,7 @@ __device__ __forceinline__ Cum6 photon_cumulants(T mu, T c, T is2, T beta)
     {
         T mg = P::wexp(fmin(lmu + (c - fp0 - (T)0.5) * is2, (T)P::kMaxExp));
         T t = 1, fphi = fp0, k = 0;
-        for (int it = 0; it < 4096; ++it) {
+        for (int it = phi_terms(p0); it > 0; --it) {
             fphi += (T)1;
             k += (T)1;
             t *= mg * P::rcp(fphi);
@@ -762,7 +769,8 @@ static __device__ __noinline__ double photon_record64(double mu, double c, doubl
     double dn = inv * ::exp(fmin(-(c - fp0 + 0.5) * is2, 600.0));
     double S[13] = {1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     double tu = 1.0, td = 1.0;
-    for (int k = 1; k < 4096; ++k) {
+    const int kend = phi_terms(p0);
+    for (int k = 1; k < kend; ++k) {
         tu *= up * rcp_count(p0 + k);
         td *= dn * (double)max(p0 - k + 1, 0);
         up *= beta;
@@ -840,7 +848,7 @@ __device__ __forceinline__ double loglik64(double mu, double c, double is2, doub
     {
         double mg = ::exp(fmin(lmu + (c - fp0 - 0.5) * is2, 700.0));
         double t = 1.0, fphi = fp0;
-        for (int it = 0; it < 4096; ++it) {
+        for (int it = phi_terms(p0); it > 0; --it) {
             fphi += 1.0;
             t *= mg / fphi;
             mg *= beta;
@@ -879,7 +887,8 @@ __device__ __forceinline__ double loglik_sum64(double mu, double mu_r, double c,
     double dn = inv * ::exp(fmin(-(c - fp0 + 0.5) * is2, 600.0));
     double S[7] = {1, 0, 0, 0, 0, 0, 0};
     double tu = 1.0, td = 1.0;
-    for (int k = 1; k < 4096; ++k) {
+    const int kend = phi_terms(p0);
+    for (int k = 1; k < kend; ++k) {
         tu *= up * rcp_count(p0 + k);
         td *= dn * (double)max(p0 - k + 1, 0);
         up *= beta;
