@@ -432,6 +432,39 @@ __device__ __forceinline__ double rcp_count(int k)
 // sums run outward from phi0 (a Newton estimate of the mode) with term
 // ratios updated multiplicatively (the Gaussian factor by exp(-1/s^2) per
 // step) until terms fall below kEps of the running sum.
+//
+// A change of many standard deviations of the photon posterior puts the weight
+// of the second sum so far out that r^k overflows before the first sum's terms
+// end.  There (dl_far64) the second sum has terms of its own, t r^k by
+// recurrence, rescaled as they grow.  (Double chains; a float chain reports the
+// update as not finite: the call would spill registers in its window loops.)
+static __device__ __noinline__ double dl_far64(double mu, double x, double c, double is2, double beta)
+{
+    const int p0 = photon_mode((float)mu, (float)c, (float)is2);
+    const double fp0 = (double)p0, d = x / mu, r = 1.0 + d, kEps = 1.3877787807814457e-17;
+    double B = 1.0, Bp = 1.0, off = 0.0;     // the sums at mu and mu + x, the second in units of exp(off)
+    auto side = [&](bool up, double ratio, double q) {
+        double t = 1.0, tp = ::exp(-off);
+        for (int k = 1; k < 1 << 24 && (up || k <= p0); ++k) {
+            const double f = up ? ratio / (fp0 + (double)k) : ratio * (fp0 - (double)(k - 1));
+            ratio *= beta;
+            t *= f;
+            tp *= f * q;
+            B += t;
+            Bp += tp;
+            if (tp > 1e200) {
+                tp *= 1e-200;
+                Bp *= 1e-200;
+                off += 460.51701859880913679;   // log 1e200
+            }
+            if (!(t >= kEps * B) && !(tp >= kEps * Bp)) break;   // (also where a term is no number)
+        }
+    };
+    side(true, mu * ::exp(fmin((c - fp0 - 0.5) * is2, 600.0)), r);
+    side(false, ::exp(fmin(-(c - fp0 + 0.5) * is2, 600.0)) / mu, 1.0 / r);
+    return -x + fp0 * ::log1p(d) + (::log(Bp) + off - ::log(B));
+}
+
 template <typename T>
 __device__ __forceinline__ T dl_pixel(T mu, T x, T c, T is2, T beta, bool& bad)
 {
@@ -522,7 +555,10 @@ __device__ __forceinline__ T dl_pixel(T mu, T x, T c, T is2, T beta, bool& bad)
             D = fma(t, e, D);
         }
     }
-    return -x + fp0 * P::log1p(d) + P::log1p(D * P::rcp(B));
+    const T y = -x + fp0 * P::log1p(d) + P::log1p(D * P::rcp(B));
+    if constexpr (sizeof(T) == 8)
+        if (!(fabs(y) <= P::kMaxFinite)) return dl_far64(mu, x, c, is2, beta);
+    return y;
 }
 
 // ------------------------------------------ photon-posterior cumulant cache

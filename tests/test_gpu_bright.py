@@ -56,7 +56,7 @@ def test_log_posterior_of_bright_noisy_frames(level, precision):
     s.close()
 
 
-@pytest.mark.parametrize("level", [4e5])
+@pytest.mark.parametrize("level", [4e5, 4e6])
 def test_likelihood_changes_of_bright_noisy_pixels(level):
     mu, p = _problem(level)
     s = bdecon.Sampler(p, precision=bdecon.BDECON_FP64, max_sweeps=4)
