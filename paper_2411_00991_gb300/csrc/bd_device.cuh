@@ -802,7 +802,7 @@ static __device__ __noinline__ double photon_record64(double mu, double c, doubl
     const double fp0 = (double)p0, inv = 1.0 / mu;
     // first term ratios: T_{p0+1}/T_p0 = up / (p0 + 1), T_{p0-1}/T_p0 = dn p0
     double up = mu * ::exp(fmin((c - fp0 - 0.5) * is2, 600.0));
-    double dn = inv * ::exp(fmin(-(c - fp0 + 0.5) * is2, 600.0));
+    double dn = p0 > 0 ? inv * ::exp(fmin(-(c - fp0 + 0.5) * is2, 600.0)) : 0.0;   // (0 inf otherwise, at the smallest mu)
     double S[13] = {1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     double tu = 1.0, td = 1.0;
     const int kend = phi_terms(p0);
@@ -920,7 +920,7 @@ __device__ __forceinline__ double loglik_sum64(double mu, double mu_r, double c,
     const int p0 = photon_mode((float)mu_r, (float)c, (float)is2);
     const double fp0 = (double)p0, inv = 1.0 / mu_r;
     double up = mu_r * ::exp(fmin((c - fp0 - 0.5) * is2, 600.0));
-    double dn = inv * ::exp(fmin(-(c - fp0 + 0.5) * is2, 600.0));
+    double dn = p0 > 0 ? inv * ::exp(fmin(-(c - fp0 + 0.5) * is2, 600.0)) : 0.0;   // (0 inf otherwise, at the smallest mu)
     double S[7] = {1, 0, 0, 0, 0, 0, 0};
     double tu = 1.0, td = 1.0;
     const int kend = phi_terms(p0);

@@ -1,4 +1,4 @@
-"""Bright pixels behind large read noise.
+"""Bright pixels behind large read noise, and the smallest expected images.
 
 With 4e5..4e6 photons a pixel and a read noise of as many photons^2 the photon
 posterior spreads over 4.5e2..1.4e3 counts, so a sum to 2^-56 of its mode runs over
@@ -69,4 +69,22 @@ def test_likelihood_changes_of_bright_noisy_pixels(level):
             ref = _change(float(p.image.flat[i]), 1.0 / level, m, new - m)
             # 28 sqrt(level) terms' logarithms, and the difference of terms of the size of |new - m|
             assert ok and abs(dl - ref) <= 1e-12 * abs(new - m) + 1e-16 * 28 * math.sqrt(level) * level ** 0.5, (i, d, dl, ref)
+    s.close()
+
+
+def test_log_posterior_at_the_smallest_expected_image():
+    rng = np.random.default_rng(3)
+    # an offset of a photon too much, 0.03 photons of read noise: the first ratio of
+    # the terms below the mode, which is 0 and has none, overflows
+    img = (0.01 * rng.normal(size=(6, 7)) - 1.0).astype(np.float32)
+    p = synth.Problem(image=img, psf=np.ones((1, 1)), gain=1.0, offset=0.0, var=1e-3, stride=1, seed=1, refresh_every=0)
+    s = bdecon.Sampler(p, precision=bdecon.BDECON_FP64, max_sweeps=4)
+    for v in (1e-10, 1e-120, 1e-140):
+        rho = np.full((6, 7), v) * (1 + 0.01 * rng.random((6, 7)))
+        s.set_state(rho, 0)
+        ref = O.Oracle(p).log_posterior(rho)
+        assert abs(s.log_posterior() - ref) <= 1e-12 * abs(ref)
+        new = 1.1 * rho.flat[5]
+        ok, dl, _ = s.delta(5, new)
+        assert ok and abs(dl + (new - rho.flat[5])) <= 1e-12 * new      # no photon: l = -mu
     s.close()
